@@ -79,6 +79,8 @@ struct AllocParams {
     int weight_kind;   // QSTATE_WEIGHT_*
     int C;             // write-back period (write-back factor weight)
     int shuf_a, shuf_b;   // shuffled-decay bijection u -> (shuf_a u + shuf_b) mod units
+    int ngroups, gshift, above_min;   // set by launch_alloc: normalisation groups, log2 of their
+                                      // size (-1: no power of two), total - units bmin
     const float* ema_s;
     const float* ema_r;
     const float* range;
