@@ -268,7 +268,8 @@ int qstate_scan_host(const qstate_cfg* cfg, qstate_buf* ping, qstate_buf* pong,
                      void* copy_stream);
 
 /* Unquantised reference path: Eq. (1) on a dense FP32 state S (device, (B, H, dk, dv), in/out)
- * for tokens [t_begin, t_end), the state round-tripping through memory every C tokens. */
+ * for tokens [t_begin, t_end).  The state is read and written once per call: FP32 values do not
+ * change on their way through memory, so the result does not depend on C. */
 int qstate_scan_fp32(const qstate_cfg* cfg, float* S, const qstate_inputs* x, int32_t t_begin,
                      int32_t t_end, float* o, void* stream);
 

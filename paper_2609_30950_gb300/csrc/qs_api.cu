@@ -878,13 +878,11 @@ int qstate_scan_fp32(const qstate_cfg* cfg, float* S, const qstate_inputs* x, in
     p.dense_in = S;
     p.dense_out = S;
     p.o = o;
-    for (int t0 = t_begin; t0 < t_end; t0 += cfg->C) {
-        p.t_begin = t0;
-        p.t_end = t0 + cfg->C < t_end ? t0 + cfg->C : t_end;
-        e = launch_step_any(*cfg, 0, 0, p, static_cast<cudaStream_t>(stream));
-        if (e != cudaSuccess) return cuda_fail(e, "fp32 write-back kernel");
-    }
-    return QSTATE_OK;
+    p.t_begin = t_begin;
+    p.t_end = t_end;
+    if (t_begin == t_end) return QSTATE_OK;
+    e = launch_scan_fp32(cfg->dk, cfg->dv, p, static_cast<cudaStream_t>(stream));
+    return e == cudaSuccess ? QSTATE_OK : cuda_fail(e, "fp32 recurrence kernel");
 }
 
 int qstate_check(void* stream) {

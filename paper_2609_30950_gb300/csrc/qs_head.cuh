@@ -1,7 +1,6 @@
 // qs_head.cuh -- write-back kernel for the head allocation unit (sm_103a): one width per head and
 // one FP16 step per scale group of 32 key rows x 1 value column (Sec. 3, "Allocation units";
-// Gated DeltaNet).  Also serves pack (dense -> packed) and unpack (packed -> dense) for this unit;
-// the dense reference path runs the general kernel.
+// Gated DeltaNet).  Also serves pack (dense -> packed) and unpack (packed -> dense) for this unit.
 //
 // One CTA of NW warps per (batch element, head).  Warp w owns row block w / NCS (32 key rows,
 // exactly one scale-group row) and column slice w % NCS (CS value columns); lane l owns the CPL

@@ -18,8 +18,7 @@
 //      per row, into a shared table; then per row the squared-error search over the candidates,
 //      codes, and the row's bits OR-ed into a zeroed shared staging row; finally one vector
 //      store of the head's new region and coalesced stores of scales / factors / ranges.
-// The same template serves pack (dense -> packed, no tokens), unpack (packed -> dense) and the
-// unquantised reference path (dense -> dense).
+// The same template serves pack (dense -> packed, no tokens) and unpack (packed -> dense).
 #pragma once
 
 #include <type_traits>
@@ -500,8 +499,7 @@ cudaError_t launch_step_t(const qstate_cfg& cfg, const StepParams& p, cudaStream
 template <int DK, int DV>
 cudaError_t launch_step_shape(const qstate_cfg& cfg, int src_packed, int dst_packed,
                               const StepParams& p, cudaStream_t stream) {
-    // the allocation unit only shapes packing: dense -> dense runs the row-unit instance
-    const bool head = cfg.unit_kind == QSTATE_UNIT_HEAD && (src_packed || dst_packed);
+    const bool head = cfg.unit_kind == QSTATE_UNIT_HEAD;
     if (head) {   // head unit: the kernel whose lanes own whole scale groups
         if constexpr (HeadGeom<DK, DV>::ok) {
             // a write-back whose per-head arrays are 16-byte aligned: the persistent kernel,
@@ -522,7 +520,6 @@ cudaError_t launch_step_shape(const qstate_cfg& cfg, int src_packed, int dst_pac
     QS_CASE(true, true)
     QS_CASE(false, true)
     QS_CASE(true, false)
-    QS_CASE(false, false)
 #undef QS_CASE
     return cudaErrorInvalidValue;
 }
