@@ -1,5 +1,6 @@
-// qs_step_impl.cuh -- general write-back kernel of libqstate for the row allocation unit (sm_103a);
-// the head unit has its own kernel (qs_head.cuh).
+// qs_step_impl.cuh -- write-back kernel of libqstate for the row allocation unit where buffers are not
+// 16-byte aligned (sm_103a; aligned ones take qs_wb_row.cuh), and the dispatch of write-back, pack and
+// unpack by state shape and unit.
 //
 // One CTA per (batch element, head), 8 warps.  Warp w owns key rows [w*RPW, (w+1)*RPW); lane
 // l owns value columns [l*CPL, (l+1)*CPL) of each of them, so one row is handled by one warp
@@ -18,13 +19,13 @@
 //      per row, into a shared table; then per row the squared-error search over the candidates,
 //      codes, and the row's bits OR-ed into a zeroed shared staging row; finally one vector
 //      store of the head's new region and coalesced stores of scales / factors / ranges.
-// The same template serves pack (dense -> packed, no tokens) and unpack (packed -> dense).
 #pragma once
 
 #include <type_traits>
 
 #include "qs_common.cuh"
 #include "qs_head.cuh"
+#include "qs_pack_row.cuh"
 
 namespace qs {
 
@@ -88,7 +89,7 @@ __device__ __forceinline__ void or_codes(uint32_t* words, int lane, int w, const
     if (hi) atomicOr(words + idx + 2, hi);
 }
 
-template <int DK, int DV, bool SRC_PACKED, bool DST_PACKED>
+template <int DK, int DV>
 __global__ void __launch_bounds__(256, 2) step_kernel(const StepParams p) {
     constexpr int NW = 8, RPW = DK / NW, CPL = DV / 32;
     using Sm = StepSmem<DK, DV>;
@@ -101,8 +102,7 @@ __global__ void __launch_bounds__(256, 2) step_kernel(const StepParams p) {
     const int bh = blockIdx.x, b = bh / p.H, h = bh - b * p.H;
     const size_t ubase = static_cast<size_t>(bh) * DK;
     const size_t gbase = static_cast<size_t>(bh) * NSG;
-    const bool has_tokens = p.t_end > p.t_begin;
-    const bool stats = has_tokens && p.ema_s != nullptr;
+    const bool stats = p.ema_s != nullptr;
 
     // ---- 1. metadata ---------------------------------------------------------------------
     if (tid == 0) sm.flag = 0;
@@ -111,14 +111,10 @@ __global__ void __launch_bounds__(256, 2) step_kernel(const StepParams p) {
         const int w = tid - 32;
         sm.inv_n[w] = w >= 2 ? __frcp_rn(static_cast<float>((1 << (w - 1)) - 1)) : 0.0f;
     }
-    if (SRC_PACKED) {
-        for (int i = tid; i < DK; i += 256) sm.w_in[i] = p.in_widths[ubase + i];
-        for (int g = tid; g < NSG; g += 256) sm.scale_in[g] = f16_value(p.in_scales[gbase + g]);
-    }
-    if (DST_PACKED) {
-        for (int i = tid; i < DK; i += 256) sm.w_out[i] = p.out_widths[ubase + i];
-        for (int g = tid; g < NSG; g += 256) sm.fidx_in[g] = p.in_fidx ? p.in_fidx[gbase + g] : 15;
-    }
+    for (int i = tid; i < DK; i += 256) sm.w_in[i] = p.in_widths[ubase + i];
+    for (int g = tid; g < NSG; g += 256) sm.scale_in[g] = f16_value(p.in_scales[gbase + g]);
+    for (int i = tid; i < DK; i += 256) sm.w_out[i] = p.out_widths[ubase + i];
+    for (int g = tid; g < NSG; g += 256) sm.fidx_in[g] = p.in_fidx[gbase + g];
     if (stats) {
         for (int i = tid; i < DK; i += 256) {
             sm.ms[i] = p.ema_s[ubase + i];
@@ -126,7 +122,7 @@ __global__ void __launch_bounds__(256, 2) step_kernel(const StepParams p) {
         }
     }
     __syncthreads();
-    if ((warp == 0 && SRC_PACKED) || (warp == 1 && DST_PACKED)) {
+    if (warp < 2) {
         const uint8_t* wa = warp == 0 ? sm.w_in : sm.w_out;
         int* off = warp == 0 ? sm.off_in : sm.off_out;
         constexpr int PER = DK / 32;
@@ -159,7 +155,7 @@ __global__ void __launch_bounds__(256, 2) step_kernel(const StepParams p) {
                 atomicExch(&sm.flag, 1);
         }
     }
-    if (SRC_PACKED && tid >= 64 && tid < 64 + DK) {
+    if (tid >= 64 && tid < 64 + DK) {
         // per-row dequantisation x = (float(u) - A) S + Bc: w >= 2 -> (q) Delta; w = 1 -> +-m;
         // w = 0 -> 0 (float(u) is 2^23 + u built from the code bits)
         const int i = tid - 64;
@@ -177,7 +173,7 @@ __global__ void __launch_bounds__(256, 2) step_kernel(const StepParams p) {
 
     // ---- 2. stage the source rows in shared memory ----------------------------------------
     using Vec = typename std::conditional<DV == 128, uint4, uint2>::type;
-    if (SRC_PACKED) {
+    {
         const int nbytes = sm.off_in[DK];
         const Vec* src = reinterpret_cast<const Vec*>(
             p.in_payload + static_cast<size_t>(b) * p.region_bytes + p.in_head_off[bh]);
@@ -193,33 +189,17 @@ __global__ void __launch_bounds__(256, 2) step_kernel(const StepParams p) {
 #pragma unroll
     for (int r = 0; r < RPW; ++r) {
         const int i = warp * RPW + r;
-        if (SRC_PACKED) {
-            const int w = sm.w_in[i];
-            uint32_t u[CPL];
-            extract_codes<CPL>(pay + sm.off_in[i], lane, w, u);
-            const float A = sm.deqA[i], S = sm.deqS[i], Bc = sm.deqB[i];
+        uint32_t u[CPL];
+        extract_codes<CPL>(pay + sm.off_in[i], lane, sm.w_in[i], u);
+        const float A = sm.deqA[i], S = sm.deqS[i], Bc = sm.deqB[i];
 #pragma unroll
-            for (int c = 0; c < CPL; ++c)
-                x[r][c] = fmaf(__fsub_rn(__uint_as_float(kTwo23Bits | u[c]), A), S, Bc);
-        } else if (p.dense_in != nullptr) {
-            const float* src = p.dense_in + (static_cast<size_t>(bh) * DK + i) * DV + lane * CPL;
-            if (CPL == 4) {
-                const float4 t = *reinterpret_cast<const float4*>(src);
-                x[r][0] = t.x; x[r][1] = t.y; x[r][CPL > 2 ? 2 : 0] = t.z; x[r][CPL > 3 ? 3 : 0] = t.w;
-            } else {
-                const float2 t = *reinterpret_cast<const float2*>(src);
-                x[r][0] = t.x; x[r][1] = t.y;
-            }
-        } else {
-#pragma unroll
-            for (int c = 0; c < CPL; ++c) x[r][c] = 0.0f;
-        }
+        for (int c = 0; c < CPL; ++c)
+            x[r][c] = fmaf(__fsub_rn(__uint_as_float(kTwo23Bits | u[c]), A), S, Bc);
     }
-    if (SRC_PACKED) __syncthreads();   // the staging buffer is reused for the output rows
-    if (DST_PACKED) {                  // zero the output rows: codes are OR-ed in
+    __syncthreads();   // the staging buffer is reused for the output rows
+    {                  // zero the output rows: codes are OR-ed in
         const int nz = (sm.off_out[DK] + 16) / 16;
         for (int i = tid; i < nz; i += 256) reinterpret_cast<uint4*>(pay)[i] = make_uint4(0, 0, 0, 0);
-        if (!has_tokens) __syncthreads();
     }
 
     // ---- 4. tokens of this write-back interval (Eq. 1) --------------------------------------
@@ -343,7 +323,7 @@ __global__ void __launch_bounds__(256, 2) step_kernel(const StepParams p) {
     }
 
     // ---- 5. write-back ------------------------------------------------------------------------
-    if (DST_PACKED) {
+    {
         const bool refit = (p.fit_every <= 1) || ((p.w_index + h) % p.fit_every == 0);
         {
             // (a) row ranges (and 1-bit means) by warp reductions
@@ -461,18 +441,6 @@ __global__ void __launch_bounds__(256, 2) step_kernel(const StepParams p) {
         }
         if (p.range != nullptr)
             for (int i = tid; i < DK; i += 256) p.range[ubase + i] = sm.rowR[i];
-    } else if (p.dense_out != nullptr) {
-#pragma unroll
-        for (int r = 0; r < RPW; ++r) {
-            const int i = warp * RPW + r;
-            float* dst = p.dense_out + (static_cast<size_t>(bh) * DK + i) * DV + lane * CPL;
-            if (CPL == 4) {
-                *reinterpret_cast<float4*>(dst) =
-                    make_float4(x[r][0], x[r][1], x[r][CPL > 2 ? 2 : 0], x[r][CPL > 3 ? 3 : 0]);
-            } else {
-                *reinterpret_cast<float2*>(dst) = make_float2(x[r][0], x[r][1]);
-            }
-        }
     }
     if (stats) {
         for (int i = tid; i < DK; i += 256) {
@@ -482,11 +450,10 @@ __global__ void __launch_bounds__(256, 2) step_kernel(const StepParams p) {
     }
 }
 
-template <int DK, int DV, bool SRC_PACKED, bool DST_PACKED>
+template <int DK, int DV>
 cudaError_t launch_step_t(const qstate_cfg& cfg, const StepParams& p, cudaStream_t stream) {
-    auto kern = step_kernel<DK, DV, SRC_PACKED, DST_PACKED>;
-    const size_t smem = sizeof(StepSmem<DK, DV>) +
-                        ((SRC_PACKED || DST_PACKED) ? static_cast<size_t>(DK) * DV * cfg.bmax / 8 + 32 : 0);
+    auto kern = step_kernel<DK, DV>;
+    const size_t smem = sizeof(StepSmem<DK, DV>) + static_cast<size_t>(DK) * DV * cfg.bmax / 8 + 32;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          static_cast<int>(smem));
     if (e != cudaSuccess) return e;
@@ -514,14 +481,9 @@ cudaError_t launch_step_shape(const qstate_cfg& cfg, int src_packed, int dst_pac
         }
         return cudaErrorInvalidValue;
     }
-#define QS_CASE(SP, DP)                                                                \
-    if ((src_packed != 0) == SP && (dst_packed != 0) == DP)                            \
-        return launch_step_t<DK, DV, SP, DP>(cfg, p, stream);
-    QS_CASE(true, true)
-    QS_CASE(false, true)
-    QS_CASE(true, false)
-#undef QS_CASE
-    return cudaErrorInvalidValue;
+    if (src_packed && dst_packed) return launch_step_t<DK, DV>(cfg, p, stream);
+    if (dst_packed) return launch_pack_row_t<DK, DV>(cfg, p, stream);
+    return launch_unpack_row_t<DK, DV>(cfg, p, stream);
 }
 
 }  // namespace qs

@@ -42,7 +42,7 @@
 
 #include <algorithm>
 
-#include "qs_common.cuh"
+#include "qs_rowquant.cuh"
 #include "qs_chunk.cuh"   // the chunked form of the interval
 
 namespace qs {
@@ -69,9 +69,8 @@ template <int DK, int DV, int NW>
 struct WbGeom {
     static constexpr int RPW = DK / NW;       // update layout: rows per warp
     static constexpr int CPL = DV / 32;       // update layout: columns per lane
-    static constexpr int TPR = DV / 32;       // row layout: lanes per row
-    static constexpr int RPB = 32 / TPR;      // row layout: rows per warp
-    static constexpr int KPT = kNFit / TPR;   // candidate steps each lane of a row prepares
+    static constexpr int TPR = RowQuant<DV>::TPR;   // row layout: lanes per row
+    static constexpr int RPB = RowQuant<DV>::RPB;   // row layout: rows per warp
 };
 
 template <int DK, int DV, int NW>
@@ -151,85 +150,6 @@ __device__ __forceinline__ void extract_codes_flat(const uint8_t* row, int lane,
     const uint64_t chunk = (static_cast<uint64_t>(hi) << 32) | lo;
 #pragma unroll
     for (int c = 0; c < CPL; ++c) u[c] = static_cast<uint32_t>(chunk >> (c * w)) & mask;
-}
-
-// ---- row layout: 32 consecutive codes of one row per lane ---------------------------------------
-// The lane's codes occupy the 4W bytes at byte 4 W q of the row (q = its part), a whole number of
-// words: code c of the run sits at bits [c W, c W + W) of those words.
-
-// Packing.  With t_c = fl(x_c / Delta) + kMagic (round to nearest even; its bit pattern is
-// kMagicBits + q_c), the stored code u_c = clamp(q_c + n, 0, 2n) is one add-min-relu on the bits;
-// codes are shifted into the lane's words (codes that straddle two words add their high bits to
-// the next word).
-template <int W, int C>
-__device__ __forceinline__ void run_put(uint32_t (&wd)[W], uint32_t u) {
-    constexpr int bp = C * W, k = bp >> 5, sh = bp & 31;
-    wd[k] += u << sh;
-    if constexpr (sh + W > 32) wd[k + 1] += u >> (32 - sh);
-}
-
-template <int W, int C>
-struct RunEncode {
-    __device__ __forceinline__ static void go(uint32_t (&wd)[W], const float2 (&xv)[16], float2 i2, int off, int top) {
-        const float2 t = __fadd2_rn(__fmul2_rn(xv[C / 2], i2), make_float2(kMagic, kMagic));
-        run_put<W, C>(wd, static_cast<uint32_t>(__viaddmin_s32_relu(__float_as_int(t.x), off, top)));
-        run_put<W, C + 1>(wd, static_cast<uint32_t>(__viaddmin_s32_relu(__float_as_int(t.y), off, top)));
-        RunEncode<W, C + 2>::go(wd, xv, i2, off, top);
-    }
-};
-template <int W>
-struct RunEncode<W, 32> {
-    __device__ __forceinline__ static void go(uint32_t (&)[W], const float2 (&)[16], float2, int, int) {}
-};
-
-// MAXA: alignment of the row starts (16 bytes for dv = 128, 8 for dv = 64).
-template <int NWD, int MAXA>
-__device__ __forceinline__ void store_words(uint8_t* dst, const uint32_t (&wd)[NWD]) {
-    if constexpr (NWD % 4 == 0 && MAXA >= 16) {
-#pragma unroll
-        for (int k = 0; k < NWD; k += 4)
-            *reinterpret_cast<uint4*>(dst + 4 * k) = make_uint4(wd[k], wd[k + 1], wd[k + 2], wd[k + 3]);
-    } else if constexpr (NWD % 2 == 0) {
-#pragma unroll
-        for (int k = 0; k < NWD; k += 2) *reinterpret_cast<uint2*>(dst + 4 * k) = make_uint2(wd[k], wd[k + 1]);
-    } else {
-#pragma unroll
-        for (int k = 0; k < NWD; ++k) reinterpret_cast<uint32_t*>(dst)[k] = wd[k];
-    }
-}
-
-// Quantise + pack the lane's 32 values (row of width W) to dst (4W bytes at byte 4 W q of a row
-// aligned to MAXA bytes): q = clamp(rint(x / Delta), -n, n), offset binary.
-template <int W, int MAXA>
-__device__ __forceinline__ void pack_run(const float2 (&xv)[16], float inv, uint8_t* dst) {
-    if constexpr (W == 1) {
-        // sign bit, code 1 for x < 0 (negative zero counts as positive)
-        uint32_t wd[1] = {0u};
-#pragma unroll
-        for (int c = 0; c < 16; ++c) {
-            wd[0] |= (xv[c].x < 0.0f ? 1u : 0u) << (2 * c);
-            wd[0] |= (xv[c].y < 0.0f ? 2u : 0u) << (2 * c);
-        }
-        store_words<1, MAXA>(dst, wd);
-    } else if constexpr (W >= 2) {
-        constexpr int n = (1 << (W - 1)) - 1;
-        uint32_t wd[W];
-#pragma unroll
-        for (int k = 0; k < W; ++k) wd[k] = 0u;
-        RunEncode<W, 0>::go(wd, xv, make_float2(inv, inv), n - static_cast<int>(kMagicBits), 2 * n);
-        store_words<W, MAXA>(dst, wd);
-    }
-}
-
-template <int MAXA>
-__device__ __forceinline__ void pack_row(int w, const float2 (&xv)[16], float inv, uint8_t* dst) {
-    switch (w) {
-#define QS_W(N) case N: pack_run<N, MAXA>(xv, inv, dst); break;
-        QS_W(1) QS_W(2) QS_W(3) QS_W(4) QS_W(5) QS_W(6) QS_W(7) QS_W(8)
-        QS_W(9) QS_W(10) QS_W(11) QS_W(12) QS_W(13) QS_W(14) QS_W(15) QS_W(16)
-#undef QS_W
-        default: break;
-    }
 }
 
 // Issue the asynchronous copies of head g's metadata into stage S, by threads t = 0..nt-1 of
@@ -326,7 +246,7 @@ template <int DK, int DV, int NW, bool CHUNK = false>
 __global__ void __launch_bounds__(NW * 32, CHUNK ? 1 : 2) wb_row_kernel(const WbParams wp) {
     using Geo = WbGeom<DK, DV, NW>;
     constexpr int RPW = Geo::RPW, CPL = Geo::CPL, CP2 = CPL / 2;
-    constexpr int TPR = Geo::TPR, RPB = Geo::RPB, KPT = Geo::KPT, NB = DK / RPB;
+    constexpr int TPR = Geo::TPR, RPB = Geo::RPB, NB = DK / RPB;
     static_assert(CPL == 2 || CPL == 4, "value columns");
     static_assert(RPW >= 2 && RPW <= 16 && NW == 8, "warps");
     using Sm = WbSmem<DK, DV, NW>;
@@ -340,11 +260,7 @@ __global__ void __launch_bounds__(NW * 32, CHUNK ? 1 : 2) wb_row_kernel(const Wb
     const int T = p.T;
 
     if (tid < kNFit) sm.fitf[tid] = fit_factor(tid);
-    if (tid >= 32 && tid < 32 + 17) {
-        const int w = tid - 32;
-        const float n = w >= 2 ? static_cast<float>((1 << (w - 1)) - 1) : 0.0f;
-        sm.wc[w] = make_float4(n, w >= 2 ? __frcp_rn(n) : 0.0f, kMagic - n, kMagic + n);
-    }
+    if (tid >= 32 && tid < 32 + 17) sm.wc[tid - 32] = width_consts(tid - 32);
 
     // a contiguous block of heads per CTA
     const int g_begin = static_cast<int>(static_cast<long long>(blockIdx.x) * wp.nheads / gridDim.x);
@@ -458,49 +374,11 @@ __global__ void __launch_bounds__(NW * 32, CHUNK ? 1 : 2) wb_row_kernel(const Wb
             const float kq = warp_sum(kk * S.q[i]);
             if (lane == 0) sm.wsum[0][(tid - 64) >> 5] = kq;
         } else if (warp == 6) {
-            // Rows in order of output width, and within a width in order of the factor fitted
-            // at the previous write-back (a close predictor of this one's), any order among
-            // equals.  Widths 2..16 come first in ascending order (the narrowest rows have the
-            // longest range-factor search), then widths 1 and 0; within a width the smaller
-            // factors first (the search runs from the largest factor down, so they search
-            // longest).  The write-back claims batches of rows in this order: longest first,
-            // and the rows of a batch stop their searches at similar candidates.  A counting
-            // sort: histogram of the 17 x 16 keys, exclusive scan, ranks from the atomics.
-            constexpr int PER = DK / 32, NK = 17 * kNFit, KPL = (NK + 31) / 32;
-            int* hist = sm.rc.hist;
-            for (int k = lane; k < NK; k += 32) hist[k] = 0;
-            __syncwarp();
-            int key[PER], rank[PER];
-#pragma unroll
-            for (int jj = 0; jj < PER; ++jj) {
-                const int i = lane * PER + jj;
-                key[jj] = ((min(static_cast<int>(S.w_out[i]), 16) + 15) % 17) * kNFit + (S.fidx[i] & (kNFit - 1));
-                rank[jj] = atomicAdd(&hist[key[jj]], 1);
-            }
-            __syncwarp();
-            int cnt[KPL], sum = 0;
-#pragma unroll
-            for (int m = 0; m < KPL; ++m) {
-                const int k = lane * KPL + m;
-                cnt[m] = sum;
-                sum += k < NK ? hist[k] : 0;
-            }
-            int incl = sum;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const int n = __shfl_up_sync(kFull, incl, o);
-                if (lane >= o) incl += n;
-            }
-            __syncwarp();
-#pragma unroll
-            for (int m = 0; m < KPL; ++m) {
-                const int k = lane * KPL + m;
-                if (k < NK) hist[k] = incl - sum + cnt[m];
-            }
-            __syncwarp();
-#pragma unroll
-            for (int jj = 0; jj < PER; ++jj)
-                sm.ord_out[hist[key[jj]] + rank[jj]] = static_cast<uint8_t>(lane * PER + jj);
+            // the write-back claims batches of rows in this order: longest searches first
+            order_rows<DK>(sm.ord_out, sm.rc.hist, lane, [&](int i, int& wd, int& f) {
+                wd = S.w_out[i];
+                f = S.fidx[i];
+            });
             if (lane == 0) sm.bat_next = NW;
         }
         __syncthreads();                                                               // B2
@@ -825,100 +703,12 @@ __global__ void __launch_bounds__(NW * 32, CHUNK ? 1 : 2) wb_row_kernel(const Wb
                 for (int o = 1; o < TPR; o <<= 1) sum += __shfl_xor_sync(kFull, sum, o);
                 if (w == 1) D = f16_round(__fdiv_rn(sum, static_cast<float>(DV)));
             }
-            const float inv_n = sm.wc[w > 16 ? 0 : w].y;
+            const float4 wc = sm.wc[w > 16 ? 0 : w];
             if (refit) {
-                __syncwarp();   // the previous batch's rows are done with the candidate table
-                // the row's 16 candidate steps, KPT per lane.  The search takes approximate
-                // reciprocals; the chosen step's IEEE reciprocal is taken below for the codes.
-#pragma unroll
-                for (int kk = 0; kk < KPT; ++kk) {
-                    const int k = q * KPT + kk;
-                    const float Dk = (w >= 2 && R > 0.0f) ? cand_step(sm.fitf[k], R, inv_n) : 0.0f;
-                    float ik = 0.0f;
-                    if (Dk > 0.0f) asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(ik) : "f"(Dk));
-                    sm.rc.cand[warp][lane / TPR][k] = make_float2(ik, -Dk);
-                }
-                __syncwarp();
-                // squared error of the candidates (levels clamped at n): e = |x| - q Delta,
-                // q = min(rint(|x| / Delta), n); the smallest wins, ties to the larger factor.
-                // Candidates are taken from the largest factor down, two per round (independent
-                // work for the warp).  Every element at or above n Delta_k quantises to n, so the
-                // clipping error of the lanes' maxima is a lower bound on candidate k's error that
-                // grows as k falls: once it exceeds the best error found (with a 2^-10 margin for
-                // rounding), no smaller factor can win.  The round's second candidate is evaluated
-                // even when its bound already rules it out; it then cannot win the comparison.
-                const float lim = sm.wc[w > 16 ? 0 : w].w, nf = sm.wc[w > 16 ? 0 : w].x;
-                float mx[TPR];
-#pragma unroll
-                for (int jl = 0; jl < TPR; ++jl) mx[jl] = __shfl_sync(kFull, lmax, (lane & ~(TPR - 1)) + jl);
-                const float2 M2 = make_float2(kMagic, kMagic), nM2 = make_float2(-kMagic, -kMagic);
-                const float2* crow = sm.rc.cand[warp][lane / TPR];
-                float bsse = INFINITY;
-                int bk = kNFit - 1;
-                // each round's two candidates are loaded one round ahead
-                float2 pA = crow[kNFit - 1], pB = crow[kNFit - 2];
-#pragma unroll 1
-                for (int k = kNFit - 1; k >= 0; k -= 2) {
-                    // candidates k and k - 1 in one round (k - 1 may not exist)
-                    const bool two = k >= 1;
-                    const float2 cA = pA, cB = two ? pB : pA;
-                    if (k >= 3) {
-                        pA = crow[k - 2];
-                        pB = crow[k - 3];
-                    }
-                    const float LA = -nf * cA.y, LB = -nf * cB.y;
-                    float lbA = 0.0f;
-#pragma unroll
-                    for (int jl = 0; jl < TPR; ++jl) {
-                        const float e = fmaxf(mx[jl] - LA, 0.0f);
-                        lbA = fmaf(e, e, lbA);
-                    }
-                    const bool goA = w >= 2 && lbA <= bsse * (1.0f + 1.0f / 1024.0f);
-                    if (!__any_sync(kFull, goA)) break;
-                    const float2 iA = make_float2(cA.x, cA.x), dA = make_float2(cA.y, cA.y);
-                    const float2 iB = make_float2(cB.x, cB.x), dB = make_float2(cB.y, cB.y);
-                    float2 aA0 = make_float2(0.0f, 0.0f), aA1 = aA0, aB0 = aA0, aB1 = aA0;
-#pragma unroll
-                    for (int c = 0; c < 16; c += 2) {
-                        float2 t0 = __ffma2_rn(av[c], iA, M2);
-                        float2 t1 = __ffma2_rn(av[c + 1], iA, M2);
-                        float2 u0 = __ffma2_rn(av[c], iB, M2);
-                        float2 u1 = __ffma2_rn(av[c + 1], iB, M2);
-                        t0.x = fminf(t0.x, lim); t0.y = fminf(t0.y, lim);
-                        t1.x = fminf(t1.x, lim); t1.y = fminf(t1.y, lim);
-                        u0.x = fminf(u0.x, lim); u0.y = fminf(u0.y, lim);
-                        u1.x = fminf(u1.x, lim); u1.y = fminf(u1.y, lim);
-                        const float2 e0 = __ffma2_rn(__fadd2_rn(t0, nM2), dA, av[c]);
-                        const float2 e1 = __ffma2_rn(__fadd2_rn(t1, nM2), dA, av[c + 1]);
-                        const float2 f0 = __ffma2_rn(__fadd2_rn(u0, nM2), dB, av[c]);
-                        const float2 f1 = __ffma2_rn(__fadd2_rn(u1, nM2), dB, av[c + 1]);
-                        aA0 = __ffma2_rn(e0, e0, aA0);
-                        aA1 = __ffma2_rn(e1, e1, aA1);
-                        aB0 = __ffma2_rn(f0, f0, aB0);
-                        aB1 = __ffma2_rn(f1, f1, aB1);
-                    }
-                    float tA = (aA0.x + aA0.y) + (aA1.x + aA1.y);
-                    float tB = (aB0.x + aB0.y) + (aB1.x + aB1.y);
-#pragma unroll
-                    for (int o = 1; o < TPR; o <<= 1) {
-                        tA += __shfl_xor_sync(kFull, tA, o);
-                        tB += __shfl_xor_sync(kFull, tB, o);
-                    }
-                    if (goA && tA < bsse) {
-                        bsse = tA;
-                        bk = k;
-                    }
-                    if (two && w >= 2 && tB < bsse) {
-                        bsse = tB;
-                        bk = k - 1;
-                    }
-                }
-                if (w >= 2) {
-                    D = -sm.rc.cand[warp][lane / TPR][bk].y;
-                    fidx = bk;
-                }
+                const int bk = fit_rows<DV>(av, lmax, R, w, wc, sm.fitf, sm.rc.cand[warp][lane / TPR], lane, D);
+                if (w >= 2) fidx = bk;
             } else if (w >= 2 && R > 0.0f) {
-                D = cand_step(sm.fitf[fidx], R, inv_n);
+                D = cand_step(sm.fitf[fidx], R, wc.y);
             }
             if (q == 0) {
                 sm.rowR[i] = R;
