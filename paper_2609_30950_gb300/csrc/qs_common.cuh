@@ -46,6 +46,32 @@ __device__ __forceinline__ float fit_factor(int k) {
 __device__ __forceinline__ float cand_step(float f, float R, float inv_n) {
     return f16_round(__fmul_rn(__fmul_rn(f, R), inv_n));
 }
+// Rounding and clamping a magnitude to its level in one operation.  In [1/2, 1) floats lie 2^-24
+// apart, so fma(y, 2^-24, 1 - n 2^-24), saturated to at most 1, is 1 - (n - q) 2^-24 with
+// q = min(rint(y), n) for y >= 0 (n < 2^23; exact halves go to the odd of two levels, n being odd):
+// one FMA-pipe operation, where a rounding add and a minimum took one and a slot of the half-rate
+// pipe of minima.  Less that constant it is q 2^-24, exactly.
+constexpr float kLevelUlp = 0x1p-24f;
+__device__ __forceinline__ float level_offset(float n) { return __fmaf_rn(-n, kLevelUlp, 1.0f); }
+__device__ __forceinline__ float round_level(float a, float inv_ulp, float offset) {
+    float t;
+    asm("fma.rn.sat.f32 %0, %1, %2, %3;" : "=f"(t) : "f"(a), "f"(inv_ulp), "f"(offset));
+    return t;
+}
+
+// Two candidate steps as the range search takes them, (2^24 Delta, approximate 2^-24 / Delta) each (0
+// for a zero step); sR = f R for two factors, or one factor's for two groups, R >= 0.  Both scalings
+// are exact: Delta has 11 significant bits and stays far inside FP32's range.
+__device__ __forceinline__ void cand_pair(float2 fR, float inv_n, float2& d_ulp, float2& inv_ulp) {
+    const float2 s = __fmul2_rn(fR, make_float2(inv_n, inv_n));
+    const float2 D = __half22float2(__floats2half2_rn(fminf(s.x, 65504.0f), fminf(s.y, 65504.0f)));
+    d_ulp = __fmul2_rn(D, make_float2(1.0f / kLevelUlp, 1.0f / kLevelUlp));
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(inv_ulp.x) : "f"(d_ulp.x));
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(inv_ulp.y) : "f"(d_ulp.y));
+    inv_ulp.x = d_ulp.x > 0.0f ? inv_ulp.x : 0.0f;
+    inv_ulp.y = d_ulp.y > 0.0f ? inv_ulp.y : 0.0f;
+}
+
 __device__ __forceinline__ float step_rcp(float D) { return D == 0.0f ? 0.0f : __frcp_rn(D); }
 
 // clamp(rint(x * inv), -n, n) in the magic domain: returns kMagic + q (exact integer float).

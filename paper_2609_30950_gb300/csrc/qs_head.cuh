@@ -73,6 +73,16 @@ __device__ __forceinline__ void hv_set(float& v, int, float s) { v = s; }
 __device__ __forceinline__ float2 hv_abs(float2 v) { return make_float2(fabsf(v.x), fabsf(v.y)); }
 __device__ __forceinline__ float hv_abs(float v) { return fabsf(v); }
 
+// The step of factor f for the lane's groups of ranges R, as the range search takes it (cand_pair).
+__device__ __forceinline__ void head_cand(float f, float2 R, float inv_n, float2& d_ulp, float2& inv_ulp) {
+    cand_pair(__fmul2_rn(make_float2(f, f), R), inv_n, d_ulp, inv_ulp);
+}
+__device__ __forceinline__ void head_cand(float f, float R, float inv_n, float& d_ulp, float& inv_ulp) {
+    d_ulp = cand_step(f, R, inv_n) * (1.0f / kLevelUlp);
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(inv_ulp) : "f"(d_ulp));
+    inv_ulp = d_ulp > 0.0f ? inv_ulp : 0.0f;
+}
+
 template <int DK, int DV, bool SRC_PACKED, bool DST_PACKED>
 __global__ void __launch_bounds__(HeadGeom<DK, DV>::NT, 2) head_kernel(const StepParams p) {
     using G = HeadGeom<DK, DV>;
@@ -322,21 +332,14 @@ __global__ void __launch_bounds__(HeadGeom<DK, DV>::NT, 2) head_kernel(const Ste
                 best[c] = INFINITY;
                 fidx[c] = kNFit - 1;
             }
-            const float lim = kMagic + nf;
-            const V M2 = hv_bc<V>(kMagic), nM2 = hv_bc<V>(-kMagic);
+            const float off = level_offset(nf), nulp = nf * kLevelUlp;
+            const V noff = hv_bc<V>(-off);
             // Candidates k and k - 1 per round (independent work for the lane); the second is
             // evaluated even when its bound already rules it out, and then cannot win.
             auto cand = [&](int k, V& iv, V& nd) {
-                const float f = sm.fitf[k];
-#pragma unroll
-                for (int c = 0; c < CPL; ++c) {
-                    const float R = hv_get(Rg, c);
-                    const float Dk = R > 0.0f ? cand_step(f, R, inv_n) : 0.0f;
-                    float ik = 0.0f;
-                    if (Dk > 0.0f) asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(ik) : "f"(Dk));
-                    hv_set(iv, c, ik);
-                    hv_set(nd, c, -Dk);
-                }
+                V d;
+                head_cand(sm.fitf[k], Rg, inv_n, d, iv);
+                nd = hv_mul(d, hv_bc<V>(-1.0f));
             };
 #pragma unroll 1
             for (int k = kNFit - 1; k >= 0; k -= 2) {
@@ -348,7 +351,7 @@ __global__ void __launch_bounds__(HeadGeom<DK, DV>::NT, 2) head_kernel(const Ste
 #pragma unroll
                 for (int c = 0; c < CPL; ++c) {
                     const float R = hv_get(Rg, c);
-                    const float e = fmaxf(R + nf * hv_get(ndA, c), 0.0f);
+                    const float e = fmaxf(R + nulp * hv_get(ndA, c), 0.0f);
                     go[c] = R > 0.0f && e * e <= best[c] * (1.0f + 1.0f / 1024.0f);
                     any |= go[c];
                 }
@@ -356,14 +359,14 @@ __global__ void __launch_bounds__(HeadGeom<DK, DV>::NT, 2) head_kernel(const Ste
                 V aA = hv_bc<V>(0.0f), aB = hv_bc<V>(0.0f);
 #pragma unroll
                 for (int r = 0; r < 32; ++r) {
-                    V tA = hv_fma(x[r], ivA, M2), tB = hv_fma(x[r], ivB, M2);
+                    V tA, tB;
 #pragma unroll
                     for (int c = 0; c < CPL; ++c) {
-                        hv_set(tA, c, fminf(hv_get(tA, c), lim));
-                        hv_set(tB, c, fminf(hv_get(tB, c), lim));
+                        hv_set(tA, c, round_level(hv_get(x[r], c), hv_get(ivA, c), off));
+                        hv_set(tB, c, round_level(hv_get(x[r], c), hv_get(ivB, c), off));
                     }
-                    const V eA = hv_fma(hv_add(tA, nM2), ndA, x[r]);
-                    const V eB = hv_fma(hv_add(tB, nM2), ndB, x[r]);
+                    const V eA = hv_fma(hv_add(tA, noff), ndA, x[r]);
+                    const V eB = hv_fma(hv_add(tB, noff), ndB, x[r]);
                     aA = hv_fma(eA, eA, aA);
                     aB = hv_fma(eB, eB, aB);
                 }
@@ -898,22 +901,19 @@ __global__ void __launch_bounds__(HeadGeom<DK, DV>::NT, 2) head_wb_kernel(const 
                     best[c] = INFINITY;
                     fidx[c] = kNFit - 1;
                 }
-                const float lim = kMagic + nf;
-                const V M2 = hv_bc<V>(kMagic), nM2 = hv_bc<V>(-kMagic);
+                const float off = level_offset(nf), nulp = nf * kLevelUlp;
+                const V noff = hv_bc<V>(-off);
 #pragma unroll 1
                 for (int k = kNFit - 1; k >= 0; --k) {
                     const float f = sm.fitf[k];
-                    V iv, nd;
+                    V iv, d;
+                    head_cand(f, Rg, inv_n, d, iv);
+                    const V nd = hv_mul(d, hv_bc<V>(-1.0f));
                     bool go[CPL], any = false;
 #pragma unroll
                     for (int c = 0; c < CPL; ++c) {
                         const float R = hv_get(Rg, c);
-                        const float Dk = R > 0.0f ? cand_step(f, R, inv_n) : 0.0f;
-                        float ik = 0.0f;
-                        if (Dk > 0.0f) asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(ik) : "f"(Dk));
-                        hv_set(iv, c, ik);
-                        hv_set(nd, c, -Dk);
-                        const float e = fmaxf(R - nf * Dk, 0.0f);
+                        const float e = fmaxf(R - nulp * hv_get(d, c), 0.0f);
                         go[c] = R > 0.0f && e * e <= best[c] * (1.0f + 1.0f / 1024.0f);
                         any |= go[c];
                     }
@@ -921,14 +921,15 @@ __global__ void __launch_bounds__(HeadGeom<DK, DV>::NT, 2) head_wb_kernel(const 
                     V a0 = hv_bc<V>(0.0f), a1 = hv_bc<V>(0.0f);
 #pragma unroll
                     for (int r = 0; r < 32; r += 2) {
-                        V t0 = hv_fma(hv_abs(x[r]), iv, M2), t1 = hv_fma(hv_abs(x[r + 1]), iv, M2);
+                        const V m0 = hv_abs(x[r]), m1 = hv_abs(x[r + 1]);
+                        V t0, t1;
 #pragma unroll
                         for (int c = 0; c < CPL; ++c) {
-                            hv_set(t0, c, fminf(hv_get(t0, c), lim));
-                            hv_set(t1, c, fminf(hv_get(t1, c), lim));
+                            hv_set(t0, c, round_level(hv_get(m0, c), hv_get(iv, c), off));
+                            hv_set(t1, c, round_level(hv_get(m1, c), hv_get(iv, c), off));
                         }
-                        const V e0 = hv_fma(hv_add(t0, nM2), nd, hv_abs(x[r]));
-                        const V e1 = hv_fma(hv_add(t1, nM2), nd, hv_abs(x[r + 1]));
+                        const V e0 = hv_fma(hv_add(t0, noff), nd, m0);
+                        const V e1 = hv_fma(hv_add(t1, noff), nd, m1);
                         a0 = hv_fma(e0, e0, a0);
                         a1 = hv_fma(e1, e1, a1);
                     }

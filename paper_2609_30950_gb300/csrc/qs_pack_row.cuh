@@ -20,9 +20,9 @@ namespace qs {
 template <int DK, int DV>
 struct alignas(16) PackSmem {
     static constexpr int NW = 4;
-    float2 cand[NW][RowQuant<DV>::RPB][kNFit + 1];   // rows padded against bank conflicts
+    float4 cand[NW][RowQuant<DV>::RPB][RowQuant<DV>::kTable];
     float4 wc[17];
-    float fitf[kNFit];
+    alignas(8) float fitf[kNFit];
     int off[DK];
     int hist[17 * kNFit + 16];
     uint8_t w[DK], order[DK];

@@ -16,6 +16,12 @@ struct RowQuant {
     static constexpr int TPR = DV / 32;
     static constexpr int RPB = 32 / TPR;
     static constexpr int KPT = kNFit / TPR;   // candidate steps each lane of a row prepares
+    // A row's candidate table: kNFit / 2 pairs of 16 bytes.  So that the rows of a warp read one pair
+    // from different banks they are permuted by row at dv = 128, where 8 KB for 8 warps is what two
+    // CTAs per SM leave, and padded at dv = 64 (an operation less per round: Mamba-2 802 against
+    // 812 us).
+    static constexpr int kTable = kNFit / 2 + (TPR == 2 ? 1 : 0);
+    static constexpr int kSwizzle = TPR == 2 ? 0 : kNFit / 2 - 1;
 };
 
 // (n, 1/n, kMagic - n, kMagic + n) of a width, n = 2^(w-1) - 1 (0 below 2 bits).
@@ -159,8 +165,8 @@ __device__ __forceinline__ void order_rows(uint8_t* order, int* hist, int lane, 
 }
 
 // The factor search of a warp's batch: av the lane's 32 magnitudes, lmax their maximum, R the row's
-// range (equal over its lanes), w its width with constants wc; table: the row's candidates, kNFit
-// float2 of the warp's own shared memory.  Returns the row's best factor index (kNFit - 1 for
+// range (equal over its lanes), w its width with constants wc; table: the row's candidate table, in
+// the warp's own shared memory.  Returns the row's best factor index (kNFit - 1 for
 // rows below 2 bits and zero rows) and its step in D (untouched below 2 bits).  TIES: also says, in
 // `close`, whether another candidate's error lies within a relative 2^-19 (n + 2) of the best: more
 // than approximate reciprocals, one rounding instead of two before the rint, and another order
@@ -168,19 +174,18 @@ __device__ __forceinline__ void order_rows(uint8_t* order, int* hist, int lane, 
 // by 8 times that, where every element sat on a rounding boundary).
 template <int DV, bool TIES = false>
 __device__ __forceinline__ int fit_rows(const float2 (&av)[16], float lmax, float R, int w, float4 wc, const float* fitf,
-                                        float2* table, int lane, float& D, bool* close = nullptr) {
+                                        float4* table, int lane, float& D, bool* close = nullptr) {
     constexpr int TPR = RowQuant<DV>::TPR, KPT = RowQuant<DV>::KPT;
-    const int q = lane % TPR;
+    const int q = lane % TPR, sw = (lane / TPR) & RowQuant<DV>::kSwizzle;
     __syncwarp();   // the previous batch's rows are done with the candidate table
     // the row's 16 candidate steps, KPT per lane.  The search takes approximate
     // reciprocals; the chosen step's IEEE reciprocal is taken for the codes.
 #pragma unroll
-    for (int kk = 0; kk < KPT; ++kk) {
-        const int k = q * KPT + kk;
-        const float Dk = (w >= 2 && R > 0.0f) ? cand_step(fitf[k], R, wc.y) : 0.0f;
-        float ik = 0.0f;
-        if (Dk > 0.0f) asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(ik) : "f"(Dk));
-        table[k] = make_float2(ik, -Dk);
+    for (int kk = 0; kk < KPT; kk += 2) {
+        const int k = q * KPT + kk;   // even
+        float2 d, iv;
+        cand_pair(__fmul2_rn(*reinterpret_cast<const float2*>(fitf + k), make_float2(R, R)), wc.y, d, iv);
+        table[(k / 2) ^ sw] = make_float4(iv.x, -d.x, iv.y, -d.y);
     }
     __syncwarp();
     // squared error of the candidates (levels clamped at n): e = |x| - q Delta,
@@ -191,11 +196,11 @@ __device__ __forceinline__ int fit_rows(const float2 (&av)[16], float lmax, floa
     // grows as k falls: once it exceeds the best error found (with a 2^-10 margin for
     // rounding), no smaller factor can win.  The round's second candidate is evaluated
     // even when its bound already rules it out; it then cannot win the comparison.
-    const float lim = wc.w, nf = wc.x;
+    const float nf = wc.x, off = level_offset(nf), nulp = nf * kLevelUlp;
     float mx[TPR];
 #pragma unroll
     for (int jl = 0; jl < TPR; ++jl) mx[jl] = __shfl_sync(kFull, lmax, (lane & ~(TPR - 1)) + jl);
-    const float2 M2 = make_float2(kMagic, kMagic), nM2 = make_float2(-kMagic, -kMagic);
+    const float2 noff = make_float2(-off, -off);
     const bool live = w >= 2 && R > 0.0f;   // a zero row keeps the largest factor
     float bsse = INFINITY, second = INFINITY;
     int bk = kNFit - 1;
@@ -203,17 +208,13 @@ __device__ __forceinline__ int fit_rows(const float2 (&av)[16], float lmax, floa
     // the bound's margin: 2^-10, or what `close` has to see
     const float margin = TIES ? fmaxf(1.0f + 0x1p-10f, near * near) : 1.0f + 0x1p-10f;
     // each round's two candidates are loaded one round ahead
-    float2 pA = table[kNFit - 1], pB = table[kNFit - 2];
+    float4 next = table[(kNFit / 2 - 1) ^ sw];
 #pragma unroll 1
     for (int k = kNFit - 1; k >= 0; k -= 2) {
-        // candidates k and k - 1 in one round (k - 1 may not exist)
-        const bool two = k >= 1;
-        const float2 cA = pA, cB = two ? pB : pA;
-        if (k >= 3) {
-            pA = table[k - 2];
-            pB = table[k - 3];
-        }
-        const float LA = -nf * cA.y;
+        // candidates k and k - 1 in one round
+        const float2 cA = make_float2(next.z, next.w), cB = make_float2(next.x, next.y);
+        if (k >= 3) next = table[(k / 2 - 1) ^ sw];
+        const float LA = -nulp * cA.y;
         float lbA = 0.0f;
 #pragma unroll
         for (int jl = 0; jl < TPR; ++jl) {
@@ -222,23 +223,18 @@ __device__ __forceinline__ int fit_rows(const float2 (&av)[16], float lmax, floa
         }
         const bool goA = live && lbA <= bsse * margin;
         if (!__any_sync(kFull, goA)) break;
-        const float2 iA = make_float2(cA.x, cA.x), dA = make_float2(cA.y, cA.y);
-        const float2 iB = make_float2(cB.x, cB.x), dB = make_float2(cB.y, cB.y);
+        const float2 dA = make_float2(cA.y, cA.y), dB = make_float2(cB.y, cB.y);
         float2 aA0 = make_float2(0.0f, 0.0f), aA1 = aA0, aB0 = aA0, aB1 = aA0;
 #pragma unroll
         for (int c = 0; c < 16; c += 2) {
-            float2 t0 = __ffma2_rn(av[c], iA, M2);
-            float2 t1 = __ffma2_rn(av[c + 1], iA, M2);
-            float2 u0 = __ffma2_rn(av[c], iB, M2);
-            float2 u1 = __ffma2_rn(av[c + 1], iB, M2);
-            t0.x = fminf(t0.x, lim); t0.y = fminf(t0.y, lim);
-            t1.x = fminf(t1.x, lim); t1.y = fminf(t1.y, lim);
-            u0.x = fminf(u0.x, lim); u0.y = fminf(u0.y, lim);
-            u1.x = fminf(u1.x, lim); u1.y = fminf(u1.y, lim);
-            const float2 e0 = __ffma2_rn(__fadd2_rn(t0, nM2), dA, av[c]);
-            const float2 e1 = __ffma2_rn(__fadd2_rn(t1, nM2), dA, av[c + 1]);
-            const float2 f0 = __ffma2_rn(__fadd2_rn(u0, nM2), dB, av[c]);
-            const float2 f1 = __ffma2_rn(__fadd2_rn(u1, nM2), dB, av[c + 1]);
+            const float2 t0 = make_float2(round_level(av[c].x, cA.x, off), round_level(av[c].y, cA.x, off));
+            const float2 t1 = make_float2(round_level(av[c + 1].x, cA.x, off), round_level(av[c + 1].y, cA.x, off));
+            const float2 u0 = make_float2(round_level(av[c].x, cB.x, off), round_level(av[c].y, cB.x, off));
+            const float2 u1 = make_float2(round_level(av[c + 1].x, cB.x, off), round_level(av[c + 1].y, cB.x, off));
+            const float2 e0 = __ffma2_rn(__fadd2_rn(t0, noff), dA, av[c]);
+            const float2 e1 = __ffma2_rn(__fadd2_rn(t1, noff), dA, av[c + 1]);
+            const float2 f0 = __ffma2_rn(__fadd2_rn(u0, noff), dB, av[c]);
+            const float2 f1 = __ffma2_rn(__fadd2_rn(u1, noff), dB, av[c + 1]);
             aA0 = __ffma2_rn(e0, e0, aA0);
             aA1 = __ffma2_rn(e1, e1, aA1);
             aB0 = __ffma2_rn(f0, f0, aB0);
@@ -256,12 +252,12 @@ __device__ __forceinline__ int fit_rows(const float2 (&av)[16], float lmax, floa
             bsse = tA;
             bk = k;
         }
-        if (two && live && tB < bsse) {
+        if (live && tB < bsse) {
             bsse = tB;
             bk = k - 1;
         }
     }
-    if (w >= 2) D = -table[bk].y;
+    if (w >= 2) D = -reinterpret_cast<const float2*>(table + ((bk / 2) ^ sw))[bk & 1].y * kLevelUlp;
     if constexpr (TIES) *close = live && !(second > bsse * near);
     return bk;
 }

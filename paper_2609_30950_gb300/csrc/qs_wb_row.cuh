@@ -79,8 +79,7 @@ struct alignas(16) WbSmem {
     float sbuf[DK * DV];                  // FP32 state of the head (swizzled rows)
     union {
         float red[2][NW][DV];             // p and r partials per warp (token phase)
-        float2 cand[NW][32 / (DV / 32)][kNFit + 1];   // per warp and row: (1/Delta_k, -Delta_k)
-                                                      // (rows padded against bank conflicts)
+        float4 cand[NW][RowQuant<DV>::RPB][RowQuant<DV>::kTable];   // per warp and row: the candidates (fit_rows)
         int hist[17 * kNFit + 16];        // prep: counting sort of the rows (width, factor)
     } rc;
     float4 deqAS[DK];                     // (-A, -A, S, S) and (B, B): x = (2^23 + u - A) S + B,
@@ -97,7 +96,7 @@ struct alignas(16) WbSmem {
     float tbeta[2];
     float u[DV];
     float rowR[DK];
-    float fitf[kNFit];
+    alignas(8) float fitf[kNFit];
     float wsum[2][NW];                    // k.q partials per warp of rows, by buffer
     alignas(16) int off_in[DK + 4];
     alignas(16) int off_out[DK + 4];
