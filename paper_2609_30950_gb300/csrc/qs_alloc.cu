@@ -148,6 +148,7 @@ __global__ void __launch_bounds__(kThreads, 1) alloc_kernel(const __grid_constan
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, u0 = tid * UPT;
     const int J = p.bmax - p.bmin, M = p.above_min;
     int w[UPT];
+    chain_wait();
 
     if (p.uniform || M == 0) {
         // equal weights: M / N bits for every unit, and the rest to the lowest indices
@@ -466,8 +467,7 @@ static cudaError_t launch_alloc_t(const AllocParams& p, cudaStream_t stream) {
     cudaError_t e = cudaFuncSetAttribute(alloc_kernel<UPT, PLAIN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          static_cast<int>(smem));
     if (e != cudaSuccess) return e;
-    alloc_kernel<UPT, PLAIN><<<p.B, threads, smem, stream>>>(p);
-    return cudaGetLastError();
+    return launch_chained(alloc_kernel<UPT, PLAIN>, p.B, threads, smem, stream, p.early != 0, p);
 }
 
 cudaError_t launch_alloc(const AllocParams& p_in, cudaStream_t stream) {

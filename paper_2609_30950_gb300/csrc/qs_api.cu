@@ -299,7 +299,7 @@ void shuffle_params(int N, int* A, int* Bo) {
 }
 
 int run_alloc(const qstate_cfg* c, const float* ms, const float* mr, const float* range, int uniform,
-              uint8_t* widths, uint32_t* head_off, int* status, cudaStream_t st) {
+              uint8_t* widths, uint32_t* head_off, int* status, cudaStream_t st, bool early = false) {
     AllocParams a;
     std::memset(&a, 0, sizeof(a));
     a.B = c->B;
@@ -322,6 +322,7 @@ int run_alloc(const qstate_cfg* c, const float* ms, const float* mr, const float
     a.widths = widths;
     a.head_off = head_off;
     a.status = status;
+    a.early = early ? 1 : 0;
     double fact = 1.0;
     for (int k = 1; k <= 16; ++k) {
         fact *= static_cast<double>(k);
@@ -463,6 +464,62 @@ int scan_parts(const qstate_cfg* c, const qstate_inputs* x, const qstate_stats* 
         if (ok) break;
     }
     return G;
+}
+
+// qstate_step; early: its launches may begin while the one before them in the stream ends (not for the
+// chains of a partitioned scan).
+int step(const qstate_cfg* cfg, qstate_buf* in, qstate_buf* out, const qstate_inputs* x, int32_t t_begin, int32_t t_end,
+         int32_t w_index, float* o, qstate_stats* stats, void* stream, bool early) {
+    int rc = validate(cfg);
+    if (rc) return rc;
+    if (!buf_ok(in) || !buf_ok(out)) return fail(QSTATE_EINVAL, "null buffer pointer");
+    if (!stats || !stats->ema_s || !stats->ema_r || (cfg->unit_kind == QSTATE_UNIT_ROW && !stats->range))
+        return fail(QSTATE_EINVAL, "null statistics pointer");
+    if ((rc = check_inputs(cfg, x, t_begin, t_end, o))) return rc;
+    if (t_end - t_begin > cfg->C || t_end == t_begin)
+        return fail(QSTATE_EINVAL, "a write-back interval holds 1..C tokens");
+    if (x->s_code && cfg->gate_bits < 1) return fail(QSTATE_EINVAL, "s_code needs gate_bits");
+    cudaStream_t st = static_cast<cudaStream_t>(stream);
+    int* status = nullptr;
+    if ((rc = acquire_status(&status))) return rc;
+    cudaError_t e;
+    StepParams p = base_params(cfg, status);
+    set_inputs(p, x);
+    p.t_begin = t_begin;
+    p.t_end = t_end;
+    p.w_index = w_index;
+    p.in_payload = in->payload;
+    p.in_scales = in->scales;
+    p.in_widths = in->widths;
+    p.in_head_off = in->head_off;
+    p.in_fidx = in->fidx;
+    p.out_payload = out->payload;
+    p.out_scales = out->scales;
+    p.out_widths = out->widths;
+    p.out_head_off = out->head_off;
+    p.out_fidx = out->fidx;
+    p.o = o;
+    p.ema_s = stats->ema_s;
+    p.ema_r = stats->ema_r;
+    p.range = stats->range;
+    p.early = early ? 1 : 0;
+    if (cfg->alloc_mode == QSTATE_ALLOC_CURRENT) {
+        // this write-back's statistics, the allocation from them, then the write-back proper
+        if (!wb_row_eligible(*cfg, p))
+            return fail(QSTATE_EINVAL, "alloc_mode current needs 16-byte aligned buffers and fidx");
+        p.mode = 1;
+        if ((e = launch_writeback(*cfg, p, st)) != cudaSuccess) return cuda_fail(e, "statistics pass");
+        rc = run_alloc(cfg, stats->ema_s, stats->ema_r, stats->range, 0, out->widths,
+                       out->head_off, status, st, early);
+        if (rc) return rc;
+        p.mode = 2;
+        if ((e = launch_writeback(*cfg, p, st)) != cudaSuccess) return cuda_fail(e, "write-back kernel");
+        return QSTATE_OK;
+    }
+    e = launch_writeback(*cfg, p, st);
+    if (e != cudaSuccess) return cuda_fail(e, "write-back kernel");
+    return run_alloc(cfg, stats->ema_s, stats->ema_r, stats->range, 0, in->widths, in->head_off,
+                     status, st, early);
 }
 
 }  // namespace
@@ -615,55 +672,7 @@ int qstate_quant_decay_noalloc(const qstate_cfg* cfg, const float* s, int32_t T,
 int qstate_step(const qstate_cfg* cfg, qstate_buf* in, qstate_buf* out, const qstate_inputs* x,
                 int32_t t_begin, int32_t t_end, int32_t w_index, float* o, qstate_stats* stats,
                 void* stream) {
-    int rc = validate(cfg);
-    if (rc) return rc;
-    if (!buf_ok(in) || !buf_ok(out)) return fail(QSTATE_EINVAL, "null buffer pointer");
-    if (!stats || !stats->ema_s || !stats->ema_r || (cfg->unit_kind == QSTATE_UNIT_ROW && !stats->range))
-        return fail(QSTATE_EINVAL, "null statistics pointer");
-    if ((rc = check_inputs(cfg, x, t_begin, t_end, o))) return rc;
-    if (t_end - t_begin > cfg->C || t_end == t_begin)
-        return fail(QSTATE_EINVAL, "a write-back interval holds 1..C tokens");
-    if (x->s_code && cfg->gate_bits < 1) return fail(QSTATE_EINVAL, "s_code needs gate_bits");
-    cudaStream_t st = static_cast<cudaStream_t>(stream);
-    int* status = nullptr;
-    if ((rc = acquire_status(&status))) return rc;
-    cudaError_t e;
-    StepParams p = base_params(cfg, status);
-    set_inputs(p, x);
-    p.t_begin = t_begin;
-    p.t_end = t_end;
-    p.w_index = w_index;
-    p.in_payload = in->payload;
-    p.in_scales = in->scales;
-    p.in_widths = in->widths;
-    p.in_head_off = in->head_off;
-    p.in_fidx = in->fidx;
-    p.out_payload = out->payload;
-    p.out_scales = out->scales;
-    p.out_widths = out->widths;
-    p.out_head_off = out->head_off;
-    p.out_fidx = out->fidx;
-    p.o = o;
-    p.ema_s = stats->ema_s;
-    p.ema_r = stats->ema_r;
-    p.range = stats->range;
-    if (cfg->alloc_mode == QSTATE_ALLOC_CURRENT) {
-        // this write-back's statistics, the allocation from them, then the write-back proper
-        if (!wb_row_eligible(*cfg, p))
-            return fail(QSTATE_EINVAL, "alloc_mode current needs 16-byte aligned buffers and fidx");
-        p.mode = 1;
-        if ((e = launch_writeback(*cfg, p, st)) != cudaSuccess) return cuda_fail(e, "statistics pass");
-        rc = run_alloc(cfg, stats->ema_s, stats->ema_r, stats->range, 0, out->widths,
-                       out->head_off, status, st);
-        if (rc) return rc;
-        p.mode = 2;
-        if ((e = launch_writeback(*cfg, p, st)) != cudaSuccess) return cuda_fail(e, "write-back kernel");
-        return QSTATE_OK;
-    }
-    e = launch_writeback(*cfg, p, st);
-    if (e != cudaSuccess) return cuda_fail(e, "write-back kernel");
-    return run_alloc(cfg, stats->ema_s, stats->ema_r, stats->range, 0, in->widths, in->head_off,
-                     status, st);
+    return step(cfg, in, out, x, t_begin, t_end, w_index, o, stats, stream, true);
 }
 
 int qstate_scan(const qstate_cfg* cfg, qstate_buf* ping, qstate_buf* pong, const qstate_inputs* x,
@@ -683,7 +692,7 @@ int qstate_scan(const qstate_cfg* cfg, qstate_buf* ping, qstate_buf* pong, const
         int w = w_index0;
         for (int t0 = t_begin; t0 < t_end; t0 += cfg->C) {
             const int t1 = t0 + cfg->C < t_end ? t0 + cfg->C : t_end;
-            rc = qstate_step(cfg, src, dst, x, t0, t1, w++, o, stats, stream);
+            rc = step(cfg, src, dst, x, t0, t1, w++, o, stats, stream, true);
             if (rc) return rc;
             qstate_buf* tmp = src;
             src = dst;
@@ -718,7 +727,7 @@ int qstate_scan(const qstate_cfg* cfg, qstate_buf* ping, qstate_buf* pong, const
         for (int p = 0; p < G && rc == QSTATE_OK; ++p) {
             qstate_buf* src = flip ? &arr[p].pong : &arr[p].ping;
             qstate_buf* dst = flip ? &arr[p].ping : &arr[p].pong;
-            rc = qstate_step(&sub[p], src, dst, &arr[p].x, t0, t1, w, arr[p].o, &arr[p].st, ps[p]);
+            rc = step(&sub[p], src, dst, &arr[p].x, t0, t1, w, arr[p].o, &arr[p].st, ps[p], false);
         }
     }
     // join, also after a failed step, so that no partition's work is left unordered

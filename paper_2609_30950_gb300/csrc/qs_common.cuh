@@ -20,6 +20,14 @@ constexpr uint32_t kMagicBits = 0x4B400000u;
 // 2^23: the float with bits 0x4B000000 | u equals 2^23 + u for u < 2^23.
 constexpr uint32_t kTwo23Bits = 0x4B000000u;
 
+// Start of a kernel launched by launch_chained: waits until the launches before it in the stream are
+// complete and their writes visible (nothing global is touched before), then lets the one after
+// it take its place on idle SMs.
+__device__ __forceinline__ void chain_wait() {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
 // Record a QS_DEV_* condition in the status word (one per device, see qs_api.cu).
 __device__ __forceinline__ void raise_status(int* status, int bits) {
     if (status) atomicOr(status, bits);

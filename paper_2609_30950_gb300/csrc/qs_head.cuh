@@ -649,6 +649,7 @@ __global__ void __launch_bounds__(HeadGeom<DK, DV>::NT, 2) head_wb_kernel(const 
     using Vec = typename std::conditional<DV == 128, uint4, uint2>::type;
 
     if (tid < kNFit) sm.fitf[tid] = fit_factor(tid);
+    chain_wait();
     const int g_begin = static_cast<int>(static_cast<long long>(blockIdx.x) * nheads / gridDim.x);
     const int g_end = static_cast<int>(static_cast<long long>(blockIdx.x + 1) * nheads / gridDim.x);
     if (g_begin >= g_end) return;
@@ -1005,8 +1006,7 @@ cudaError_t launch_head_wb_t(const qstate_cfg& cfg, const StepParams& p, cudaStr
     if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, HeadGeom<DK, DV>::NT, smem)) != cudaSuccess) return e;
     const int nheads = cfg.B * cfg.H;
     const int grid = std::min(nheads, std::max(1, per_sm) * sms);
-    kern<<<grid, HeadGeom<DK, DV>::NT, smem, stream>>>(q, nheads);
-    return cudaGetLastError();
+    return launch_chained(kern, grid, HeadGeom<DK, DV>::NT, smem, stream, q.early != 0, q, nheads);
 }
 
 }  // namespace qs

@@ -264,10 +264,10 @@ __global__ void __launch_bounds__(NW * 32, CHUNK ? 1 : 2) wb_row_kernel(const Wb
     // a contiguous block of heads per CTA
     const int g_begin = static_cast<int>(static_cast<long long>(blockIdx.x) * wp.nheads / gridDim.x);
     const int g_end = static_cast<int>(static_cast<long long>(blockIdx.x + 1) * wp.nheads / gridDim.x);
-    if (g_begin >= g_end) return;
     uint8_t* cb = pay + ((p.stage_bytes + 32 + 15) & ~15);   // chunked form's region
     uint32_t tmem = 0, mphase = 0;
     if constexpr (CHUNK) tmem = chunk_setup(cb);
+    chain_wait();
     {
         const int h0 = g_begin % p.H;
         const int io = static_cast<int>(p.in_head_off[g_begin]);
@@ -753,8 +753,7 @@ cudaError_t launch_wb_row_t(const qstate_cfg& cfg, const StepParams& sp, cudaStr
     if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
     if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, NW * 32, smem)) != cudaSuccess) return e;
     const int grid = std::min(wp.nheads, std::max(1, per_sm) * sms);
-    kern<<<grid, NW * 32, smem, stream>>>(wp);
-    return cudaGetLastError();
+    return launch_chained(kern, grid, NW * 32, smem, stream, wp.s.early != 0, wp);
 }
 
 }  // namespace qs
