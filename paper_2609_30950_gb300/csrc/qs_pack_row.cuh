@@ -13,10 +13,10 @@ namespace qs {
 // and stores them without any exchange beyond the row's TPR lanes.  16 warps per SM: the loads of
 // some hide behind the searches of the others.
 // What bounds it: the search's FP32 work (about 36 lane-instructions per element), ahead of HBM
-// (64 KB read per head).  64 x 32 heads of 128 x 128, 4 bits: 88 us (151 MB, 1.7 TB/s); 214 us with all
+// (64 KB read per head).  64 x 32 heads of 128 x 128, 4 bits: 78 us (151 MB, 1.9 TB/s); 214 us with all
 // 16 candidates of every row in scalar arithmetic, a row spread over a warp.  Results are those of that
 // arithmetic bit for bit (each product and sum of a code rounded by itself, near ties between factors
-// decided by fit_rows_exact); without that 80 us.
+// decided by fit_rows_exact); without that it took 80 us when it took 88 with it.
 template <int DK, int DV>
 struct alignas(16) PackSmem {
     static constexpr int NW = 4;
@@ -132,7 +132,7 @@ __global__ void __launch_bounds__(128, 4) pack_row_kernel(const __grid_constant_
             if (w == 1) D = f16_round(__fdiv_rn(sum, static_cast<float>(DV)));
         }
         bool close = false;
-        const int bk = fit_rows<DV, true>(av, lmax, R, w, sm.wc[w], sm.fitf, sm.cand[warp][lane / TPR], lane, D, &close);
+        const int bk = fit_rows<DV, true>(av, m4, R, w, sm.wc[w], sm.fitf, sm.cand[warp][lane / TPR], lane, D, &close);
         if (w >= 2) fidx = bk;
         if (__any_sync(kFull, close)) {
             // near ties (a few rows in a million at 4 bits): decided in a fixed arithmetic, which

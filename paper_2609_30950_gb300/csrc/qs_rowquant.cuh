@@ -164,8 +164,8 @@ __device__ __forceinline__ void order_rows(uint8_t* order, int* hist, int lane, 
     for (int jj = 0; jj < PER; ++jj) order[hist[key[jj]] + rank[jj]] = static_cast<uint8_t>(lane * PER + jj);
 }
 
-// The factor search of a warp's batch: av the lane's 32 magnitudes, lmax their maximum, R the row's
-// range (equal over its lanes), w its width with constants wc; table: the row's candidate table, in
+// The factor search of a warp's batch: av the lane's 32 magnitudes, m4 the maxima of four
+// disjoint parts of them, R the row's range (equal over its lanes), w its width with constants wc; table: the row's candidate table, in
 // the warp's own shared memory.  Returns the row's best factor index (kNFit - 1 for
 // rows below 2 bits and zero rows) and its step in D (untouched below 2 bits).  TIES: also says, in
 // `close`, whether another candidate's error lies within a relative 2^-19 (n + 2) of the best: more
@@ -173,7 +173,7 @@ __device__ __forceinline__ void order_rows(uint8_t* order, int* hist, int lane, 
 // of the sum can change an error (a position in steps moves by at most n 2^-22, and an error
 // by 8 times that, where every element sat on a rounding boundary).
 template <int DV, bool TIES = false>
-__device__ __forceinline__ int fit_rows(const float2 (&av)[16], float lmax, float R, int w, float4 wc, const float* fitf,
+__device__ __forceinline__ int fit_rows(const float2 (&av)[16], const float (&m4)[4], float R, int w, float4 wc, const float* fitf,
                                         float4* table, int lane, float& D, bool* close = nullptr) {
     constexpr int TPR = RowQuant<DV>::TPR, KPT = RowQuant<DV>::KPT;
     const int q = lane % TPR, sw = (lane / TPR) & RowQuant<DV>::kSwizzle;
@@ -192,14 +192,35 @@ __device__ __forceinline__ int fit_rows(const float2 (&av)[16], float lmax, floa
     // q = min(rint(|x| / Delta), n); the smallest wins, ties to the larger factor.
     // Candidates are taken from the largest factor down, two per round (independent
     // work for the warp).  Every element at or above n Delta_k quantises to n, so the
-    // clipping error of the lanes' maxima is a lower bound on candidate k's error that
+    // clipping error of some of them is a lower bound on candidate k's error that
     // grows as k falls: once it exceeds the best error found (with a 2^-10 margin for
     // rounding), no smaller factor can win.  The round's second candidate is evaluated
     // even when its bound already rules it out; it then cannot win the comparison.
     const float nf = wc.x, off = level_offset(nf), nulp = nf * kLevelUlp;
-    float mx[TPR];
+    // A candidate's bound.  dv = 128: from 4 maxima of 8 elements per lane, summed over the row's
+    // lanes (about half an evaluation per row fewer than from the 4 lane maxima: KDA decode 357
+    // against 360 us per token, pack 78 against 80); made one round ahead, beside the evaluations.
+    // dv = 64: from the row's 2 lane maxima, without a sum (Mamba-2, whose wider rows stop
+    // early: 201 against 206 us).
+    float mx[2];
+    if constexpr (TPR == 2) {
+        const float lmax = fmaxf(fmaxf(m4[0], m4[1]), fmaxf(m4[2], m4[3]));
+        mx[0] = lmax;
+        mx[1] = __shfl_xor_sync(kFull, lmax, 1);
+    }
+    auto bound = [&](float d_ulp) {
+        float lb = 0.0f;
 #pragma unroll
-    for (int jl = 0; jl < TPR; ++jl) mx[jl] = __shfl_sync(kFull, lmax, (lane & ~(TPR - 1)) + jl);
+        for (int j = 0; j < (TPR == 2 ? 2 : 4); ++j) {
+            const float e = fmaxf(fmaf(nulp, d_ulp, TPR == 2 ? mx[j & 1] : m4[j]), 0.0f);
+            lb = fmaf(e, e, lb);
+        }
+        if constexpr (TPR != 2) {
+#pragma unroll
+            for (int o = 1; o < TPR; o <<= 1) lb += __shfl_xor_sync(kFull, lb, o);
+        }
+        return lb;
+    };
     const float2 noff = make_float2(-off, -off);
     const bool live = w >= 2 && R > 0.0f;   // a zero row keeps the largest factor
     float bsse = INFINITY, second = INFINITY;
@@ -209,20 +230,21 @@ __device__ __forceinline__ int fit_rows(const float2 (&av)[16], float lmax, floa
     const float margin = TIES ? fmaxf(1.0f + 0x1p-10f, near * near) : 1.0f + 0x1p-10f;
     // each round's two candidates are loaded one round ahead
     float4 next = table[(kNFit / 2 - 1) ^ sw];
+    float lbA = 0.0f;   // the first round always runs
 #pragma unroll 1
     for (int k = kNFit - 1; k >= 0; k -= 2) {
         // candidates k and k - 1 in one round
         const float2 cA = make_float2(next.z, next.w), cB = make_float2(next.x, next.y);
-        if (k >= 3) next = table[(k / 2 - 1) ^ sw];
-        const float LA = -nulp * cA.y;
-        float lbA = 0.0f;
-#pragma unroll
-        for (int jl = 0; jl < TPR; ++jl) {
-            const float e = fmaxf(mx[jl] - LA, 0.0f);
-            lbA = fmaf(e, e, lbA);
-        }
+        if constexpr (TPR == 2) lbA = bound(cA.y);
         const bool goA = live && lbA <= bsse * margin;
+        if constexpr (TPR == 2) {
+            if (k >= 3) next = table[(k / 2 - 1) ^ sw];
+        }
         if (!__any_sync(kFull, goA)) break;
+        if constexpr (TPR != 2) {
+            if (k >= 3) next = table[(k / 2 - 1) ^ sw];
+            lbA = bound(next.w);
+        }
         const float2 dA = make_float2(cA.y, cA.y), dB = make_float2(cB.y, cB.y);
         float2 aA0 = make_float2(0.0f, 0.0f), aA1 = aA0, aB0 = aA0, aB1 = aA0;
 #pragma unroll

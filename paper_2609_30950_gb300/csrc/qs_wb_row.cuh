@@ -704,7 +704,7 @@ __global__ void __launch_bounds__(NW * 32, CHUNK ? 1 : 2) wb_row_kernel(const Wb
             }
             const float4 wc = sm.wc[w > 16 ? 0 : w];
             if (refit) {
-                const int bk = fit_rows<DV>(av, lmax, R, w, wc, sm.fitf, sm.rc.cand[warp][lane / TPR], lane, D);
+                const int bk = fit_rows<DV>(av, m4, R, w, wc, sm.fitf, sm.rc.cand[warp][lane / TPR], lane, D);
                 if (w >= 2) fidx = bk;
             } else if (w >= 2 && R > 0.0f) {
                 D = cand_step(sm.fitf[fidx], R, wc.y);
