@@ -54,11 +54,11 @@ struct ChunkGeo {
     // TMEM columns: S^T (FP32, read by the products as its TF32 part hi) and lo, the block's update, the product with S_b (hi*hi part and
     // corrections), u^T hi / lo, the product (k / Dc) [a o Dc ; q o Dc]^T that gives A and M
     static constexpr uint32_t kHi = 0, kLo = 128, kUpd = 256, kDW = 384, kDWc = 416, kUHi = 448,
-                              kULo = 464, kAM = 480;
-    // The correction products of A and M (hi*lo + lo*hi) accumulate apart from hi*hi, in the
-    // update's columns: those are free from the state combine of one block to the update
-    // product of the next, and A and M are read out before that product is issued.
-    static constexpr uint32_t kAMc = kUpd;
+                              kULo = 464;
+    // hi*hi and corrections of A and M, beside each other in the update's columns: those are free
+    // from the state combine of one block to the update product of the next, and A and M are read
+    // out before that product is issued.
+    static constexpr uint32_t kAM = kUpd, kAMc = kUpd + 2 * L;
     static constexpr uint32_t kCols = 512;
     // Operand tiles (K-major core matrices, see qs_tc.cuh).  A K-chunk is padded by 16 bytes
     // where a warp writes one column of consecutive key rows, so the writes spread over all
@@ -67,13 +67,15 @@ struct ChunkGeo {
     //          M = 64 product: rows 16..63 alias the following bytes (always inside the
     //          region, read but never used), their output lanes are ignored.
     static constexpr uint32_t kLboH = L * 16 + 16, kSboH = 128;
-    //  [a o Dc ; q o Dc]: 2L rows x D, K-chunks 528 bytes apart
-    static constexpr uint32_t kLboW = 2 * L * 16 + 16, kSboW = 128;
+    //  [a o Dc ; q o Dc]: 2L rows x D of hi parts and, in the same K-chunks, 2L rows of lo
+    //          parts, K-chunks 1040 bytes apart: a product with the 4L rows gives hi*hi and hi*lo
+    //          in neighbouring columns (kDW and kDWc, kAM and kAMc) at the cost of one
+    static constexpr uint32_t kLboW = 4 * L * 16 + 16, kSboW = 128;
     //  (k o Dc_{L-1} / Dc)^T: D rows (key rows) x L (K = token)
     static constexpr uint32_t kLboU = (D / 8) * 128, kSboU = 128;
     static constexpr uint32_t kKh = (D / 4) * kLboH, kBw = (D / 4) * kLboW, kBu = (L / 4) * kLboU;
-    static constexpr uint32_t oKhHi = 0, oKhLo = kKh, oBwHi = 2 * kKh, oBwLo = 2 * kKh + kBw;
-    static constexpr uint32_t oBuHi = 2 * kKh + 2 * kBw, oBuLo = oBuHi + kBu;
+    static constexpr uint32_t oKhHi = 0, oKhLo = kKh, oBwHi = 2 * kKh, oBwLo = oBwHi + 2 * L * 16;
+    static constexpr uint32_t oBuHi = 2 * kKh + kBw, oBuLo = oBuHi + kBu;
     static constexpr uint32_t oAM = oBuLo + kBu;                  // A and M, L x L each
     static constexpr uint32_t oDall = oAM + 2 * L * L * 4;        // two buffers, by block parity
     static constexpr uint32_t oXch = oDall + 2 * D * 4;          // row preparation: the halves' exchange
@@ -90,9 +92,10 @@ struct ChunkGeo {
 static_assert(ChunkGeo::oBwHi % 16 == 0 && ChunkGeo::oBuHi % 16 == 0 && ChunkGeo::oBar % 16 == 0 &&
               ChunkGeo::oStg % 16 == 0, "tile alignment");
 // the aliased rows of the k / Dc operand (16 row groups of 128 bytes from each K-step's start)
-// stay inside the two k / Dc tiles and the first [a o Dc ; q o Dc] tile
+// stay inside the k / Dc tiles and the [a o Dc ; q o Dc] tile
 static_assert(ChunkGeo::oKhLo + (ChunkGeo::D / 8 - 1) * 2 * ChunkGeo::kLboH + ChunkGeo::kLboH + 16 * 128 <=
-              ChunkGeo::oBwLo, "aliased operand rows");
+              ChunkGeo::oBuHi, "aliased operand rows");
+static_assert(ChunkGeo::kDWc == ChunkGeo::kDW + 2 * ChunkGeo::L, "hi*hi and hi*lo columns of one product");
 
 __device__ __forceinline__ volatile uint32_t* chunk_abort_word(uint8_t* cb) {
     return reinterpret_cast<volatile uint32_t*>(cb + ChunkGeo::oBar + 20);
@@ -425,22 +428,19 @@ __device__ __forceinline__ void chunk_interval(const StepParams& p, Stage& S, fl
         // A_ts (column < L) or M_ts (column >= L)
         if (tid == 0 || tid == 32) {
             tc::fence_after_sync();
-            constexpr uint32_t idW = tc::idesc_tf32(128, 2 * L);
+            constexpr uint32_t idW = tc::idesc_tf32(128, 2 * L), idW2 = tc::idesc_tf32(128, 4 * L);
             // A and M need rows 0..L-1 of the product only: M = 64 (rows 0..15 land in lanes 0..15)
-            constexpr uint32_t idAM = tc::idesc_tf32(64, 2 * L);
+            constexpr uint32_t idAM = tc::idesc_tf32(64, 2 * L), idAM2 = tc::idesc_tf32(64, 4 * L);
             // a K-step advances the start addresses (16-byte units, bits 0-13) by two K-chunks
             constexpr uint64_t kStepW = (2 * G::kLboW) >> 4, kStepH = (2 * G::kLboH) >> 4;
             uint64_t bh = tc::smem_desc(tc::smem_addr(bw_hi), G::kLboW, G::kSboW);
-            uint64_t bl = tc::smem_desc(tc::smem_addr(bw_lo), G::kLboW, G::kSboW);
             if (tid == 0) {
 #pragma unroll
                 for (int ks = 0; ks < D / 8; ++ks) {
                     const uint32_t acc = ks > 0 ? 1u : 0u;
-                    tc::mma_tf32_ts(tmem + G::kDW, tmem + G::kHi + 8 * ks, bh, idW, acc);
-                    tc::mma_tf32_ts(tmem + G::kDWc, tmem + G::kHi + 8 * ks, bl, idW, acc);
+                    tc::mma_tf32_ts(tmem + G::kDW, tmem + G::kHi + 8 * ks, bh, idW2, acc);
                     tc::mma_tf32_ts(tmem + G::kDWc, tmem + G::kLo + 8 * ks, bh, idW, 1u);
                     bh += kStepW;
-                    bl += kStepW;
                 }
             } else {
                 uint64_t ah = tc::smem_desc(tc::smem_addr(kh_hi), G::kLboH, G::kSboH);
@@ -448,11 +448,9 @@ __device__ __forceinline__ void chunk_interval(const StepParams& p, Stage& S, fl
 #pragma unroll
                 for (int ks = 0; ks < D / 8; ++ks) {
                     const uint32_t acc = ks > 0 ? 1u : 0u;
-                    tc::mma_tf32_ss(tmem + G::kAM, ah, bh, idAM, acc);
-                    tc::mma_tf32_ss(tmem + G::kAMc, ah, bl, idAM, acc);
+                    tc::mma_tf32_ss(tmem + G::kAM, ah, bh, idAM2, acc);
                     tc::mma_tf32_ss(tmem + G::kAMc, al, bh, idAM, 1u);
                     bh += kStepW;
-                    bl += kStepW;
                     ah += kStepH;
                     al += kStepH;
                 }
