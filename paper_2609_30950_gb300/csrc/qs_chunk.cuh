@@ -78,10 +78,12 @@ struct ChunkGeo {
     static constexpr uint32_t oBuHi = 2 * kKh + kBw, oBuLo = oBuHi + kBu;
     static constexpr uint32_t oAM = oBuLo + kBu;                  // A and M, L x L each
     static constexpr uint32_t oDall = oAM + 2 * L * L * 4;        // two buffers, by block parity
-    static constexpr uint32_t oXch = oDall + 2 * D * 4;          // row preparation: the halves' exchange
+    // row preparation: the quarters' decay products; the EMA terms of quarters 0 and 2; the EMA state
+    // after the first half
+    static constexpr uint32_t oXp = oDall + 2 * D * 4, oXt = oXp + 4 * D * 4, oXm = oXt + 2 * 2 * D * 16;
     // mbarriers of the products with S_b and A / M (two arrivals) and of the update (one); the
     // TMEM address (byte 16), the abort word (byte 20) and the teardown's mbarrier (byte 24)
-    static constexpr uint32_t oBar = oXch + 2 * D * 16;
+    static constexpr uint32_t oBar = oXm + D * 8;
     // one block's token inputs, staged by cp.async: k, q, rates (FP32 per row, per head, or
     // uint8 codes) and beta (three buffers by block index mod 3: block c's solve still reads
     // its beta while block c + 2's arrives)
@@ -171,9 +173,9 @@ __device__ __forceinline__ void chunk_interval(const StepParams& p, Stage& S, fl
     using G = ChunkGeo;
     constexpr int L = G::L, D = G::D;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int sub = warp & 3, hf = warp >> 2;
+    const int sub = warp & 3, hf = warp >> 2;   // 16 warps: four for each 32 TMEM lanes
     const int jl = 32 * sub + lane;   // the TMEM lane (value column) this thread addresses
-    const int tt = tid - 128;         // index among the value-column threads (warps 4-7)
+    const int tt = hf == 1 ? tid - 128 : -1;   // index among the value-column threads (warps 4-7)
     const uint32_t tl = tmem + (static_cast<uint32_t>(32 * sub) << 16);
     uint64_t* bar = reinterpret_cast<uint64_t*>(cb + G::oBar);
     float* amA = reinterpret_cast<float*>(cb + G::oAM);
@@ -240,7 +242,7 @@ __device__ __forceinline__ void chunk_interval(const StepParams& p, Stage& S, fl
 
     // state in: S^T into TMEM (FP32 and lo); this thread's lane j, key rows of its half
 #pragma unroll 1
-    for (int i0 = 64 * hf; i0 < 64 * hf + 64; i0 += 16) {
+    for (int i0 = 32 * hf; i0 < 32 * hf + 32; i0 += 16) {
         float x[16], lo[16];
 #pragma unroll
         for (int c = 0; c < 16; ++c) {
@@ -253,22 +255,25 @@ __device__ __forceinline__ void chunk_interval(const StepParams& p, Stage& S, fl
     tc::wait_st();
     tc::fence_before_sync();
 
-    // Rows: thread (i, half hh) takes tokens 8 hh .. 8 hh + 7 of key row i.  Phase A (staged
-    // loads, decays, EMA terms, the first half's EMA recursion) of block c + 1 runs while the
-    // tensor cores work on block c; phase B (the second half's EMA recursion, cumulative decays,
-    // operand tiles) at the start of block c + 1.  The halves exchange through shared memory the
-    // first half's decay product and EMA state and the second half's decay product.
-    constexpr int LH = L / 2;
-    const int i = tid & (D - 1), hh = tid >> 7, tb = LH * hh;
-    float4* xch = reinterpret_cast<float4*>(cb + G::oXch);
+    // Rows: thread (i, quarter qt) takes tokens 4 qt .. 4 qt + 3 of key row i.  Phase A (staged
+    // loads, decays, EMA terms) of block c + 1 runs while the tensor cores work on block c, the EMA
+    // recursion over the first half's tokens beside the solve, and phase B (the second half's EMA
+    // recursion, cumulative decays, operand tiles) at the start of block c + 1.  The quarters
+    // exchange their decay products through shared memory; quarters 1 and 3 (warps 0-3 and 12-15,
+    // which neither solve nor copy) run the recursions, with the terms of quarters 0 and 2.
+    constexpr int LH = L / 4;
+    const int i = tid & (D - 1), qt = hf < 2 ? hf ^ 1 : hf, tb = LH * qt;
+    float* xp = reinterpret_cast<float*>(cb + G::oXp);
+    float4* xt = reinterpret_cast<float4*>(cb + G::oXt);
+    float2* xm = reinterpret_cast<float2*>(cb + G::oXm);
     struct RowA {
         float kk[LH], dd[LH], qv[LH], bv[LH], xs[LH], xr[LH];
     };
     auto phase_a = [&](int t0b, RowA& r) {
         const int nb = min(L, p.t_end - t0b);
         const float* sbeta = reinterpret_cast<const float*>(stg + G::sB) + (((t0b - p.t_begin) / L) % 3) * L;
-        // branch-free over the half's tokens (tokens past nb read staged bytes of earlier
-        // blocks, in bounds, and are masked), so the eight exp / expm1 chains interleave
+        // branch-free over the quarter's tokens (tokens past nb read staged bytes of earlier
+        // blocks, in bounds, and are masked), so the four exp / expm1 chains interleave
         bool bad = false;
 #pragma unroll
         for (int j = 0; j < LH; ++j) {
@@ -303,26 +308,35 @@ __device__ __forceinline__ void chunk_interval(const StepParams& p, Stage& S, fl
         float prod = 1.0f;
 #pragma unroll
         for (int j = 0; j < LH; ++j) prod = __fmul_rn(prod, r.dd[j]);
-        if (hh == 0) {
-            // the EMA recursion over the first half (from the state after the previous block)
-            float ms = stats ? S.ms[i] : 0.0f, mr = stats ? S.mr[i] : 0.0f;
-            if (stats) {
-#pragma unroll
-                for (int j = 0; j < LH; ++j) {
-                    if (j >= nb) break;
-                    if (t0b + j == 0) {
-                        ms = r.xs[j];
-                        mr = r.xr[j];
-                    } else {
-                        ms = __fadd_rn(ms, __fmul_rn(p.alpha, __fsub_rn(r.xs[j], ms)));
-                        mr = __fadd_rn(mr, __fmul_rn(p.alpha, __fsub_rn(r.xr[j], mr)));
-                    }
-                }
-            }
-            xch[i] = make_float4(prod, ms, mr, 0.0f);
-        } else {
-            xch[D + i].x = prod;
+        xp[qt * D + i] = prod;
+        if (stats && (qt & 1) == 0) {
+            xt[qt * D + i] = make_float4(r.xs[0], r.xs[1], r.xs[2], r.xs[3]);
+            xt[(qt + 1) * D + i] = make_float4(r.xr[0], r.xr[1], r.xr[2], r.xr[3]);
         }
+    };
+    // One half's EMA recursion, token by token: the even quarter's terms and then the own ones.
+    auto ema_half = [&](int t0b, const RowA& r, float& ms, float& mr) {
+        const int nb = min(L, p.t_end - t0b), tq = tb - LH;
+        const float4 s4 = xt[(qt - 1) * D + i], r4 = xt[qt * D + i];
+        const float xs[2 * LH] = {s4.x, s4.y, s4.z, s4.w, r.xs[0], r.xs[1], r.xs[2], r.xs[3]};
+        const float xr[2 * LH] = {r4.x, r4.y, r4.z, r4.w, r.xr[0], r.xr[1], r.xr[2], r.xr[3]};
+#pragma unroll
+        for (int j = 0; j < 2 * LH; ++j) {
+            if (tq + j >= nb) break;
+            if (t0b + tq + j == 0) {
+                ms = xs[j];
+                mr = xr[j];
+            } else {
+                ms = __fadd_rn(ms, __fmul_rn(p.alpha, __fsub_rn(xs[j], ms)));
+                mr = __fadd_rn(mr, __fmul_rn(p.alpha, __fsub_rn(xr[j], mr)));
+            }
+        }
+    };
+    auto first_half = [&](int t0b, const RowA& r) {   // quarter 1, a barrier after phase A
+        if (!stats || qt != 1) return;
+        float ms = S.ms[i], mr = S.mr[i];
+        ema_half(t0b, r, ms, mr);
+        xm[i] = make_float2(ms, mr);
     };
     auto phase_b = [&](int t0b, const RowA& r) {
         const int nb = min(L, p.t_end - t0b);
@@ -337,20 +351,19 @@ __device__ __forceinline__ void chunk_interval(const StepParams& p, Stage& S, fl
             sf[j] = acc;
             acc = __fmul_rn(acc, r.dd[j]);
         }
-        const float4 x0 = xch[i];
-        const float dc0 = hh == 0 ? 1.0f : x0.x;            // decay before the half
-        const float sf1 = hh == 0 ? xch[D + i].x : 1.0f;   // decay after the half, in the block
-        if (hh == 1) {
-            // the EMA state after the whole block and the block's decay (with no second-half
-            // tokens, the first half's)
-            float ms = x0.y, mr = x0.z;
-            if (stats) {
+        // decay of the block before and after the quarter
+        float dc0 = 1.0f, sf1 = 1.0f;
 #pragma unroll
-                for (int j = 0; j < LH; ++j) {
-                    if (tb + j >= nb) break;
-                    ms = __fadd_rn(ms, __fmul_rn(p.alpha, __fsub_rn(r.xs[j], ms)));
-                    mr = __fadd_rn(mr, __fmul_rn(p.alpha, __fsub_rn(r.xr[j], mr)));
-                }
+        for (int q = 0; q < 3; ++q)
+            if (q < qt) dc0 = __fmul_rn(dc0, xp[q * D + i]);
+#pragma unroll
+        for (int q = 3; q > 0; --q)
+            if (q > qt) sf1 = __fmul_rn(sf1, xp[q * D + i]);
+        if (qt == 3) {
+            // the EMA state after the whole block, and the block's decay
+            if (stats) {
+                float ms = xm[i].x, mr = xm[i].y;
+                ema_half(t0b, r, ms, mr);
                 S.ms[i] = ms;
                 S.mr[i] = mr;
             }
@@ -378,7 +391,7 @@ __device__ __forceinline__ void chunk_interval(const StepParams& p, Stage& S, fl
             *reinterpret_cast<float*>(bw_hi + ow + 16 * (L + tau)) = qth;
             *reinterpret_cast<float*>(bw_lo + ow + 16 * (L + tau)) = __fsub_rn(qt, qth);
         }
-        // (k o Dc_{L-1} / Dc)^T: row i, tokens of the half, 4 per 16-byte chunk
+        // (k o Dc_{L-1} / Dc)^T: row i, tokens of the quarter, 4 per 16-byte chunk
 #pragma unroll
         for (int c4 = 0; c4 < LH / 4; ++c4) {
             float kb[4];
@@ -407,6 +420,8 @@ __device__ __forceinline__ void chunk_interval(const StepParams& p, Stage& S, fl
         phase_a(p.t_begin, ra);
         __syncthreads();                      // the first block's exchange; its staging is read
         if (tt >= 0 && p.t_begin + L < p.t_end) issue_kqs(p.t_begin + L);
+        first_half(p.t_begin, ra);
+        __syncthreads();
     }
 
 #pragma unroll 1
@@ -478,6 +493,7 @@ __device__ __forceinline__ void chunk_interval(const StepParams& p, Stage& S, fl
         // every thread is done with the next block's staged inputs: the one after it
         if (tt >= 0 && t0 + 2 * L < p.t_end) issue_kqs(t0 + 2 * L);
 
+        if (!last) first_half(t0 + L, ra);
         if (hf == 1) {
             // u of column j, token by token: u_t = w_t v_t - (S_b^T (a o Dc))_t - sum_{s<t} A_ts u_s
             float wk[L], ck[L];
@@ -532,8 +548,9 @@ __device__ __forceinline__ void chunk_interval(const StepParams& p, Stage& S, fl
         }
         {
             // readouts of column j: o_t = (S_b^T (q o Dc))_t + sum_{s<=t} M_ts u_s, with u from
-            // its hi / lo parts in TMEM; warps 0-3 take tokens 0..7 (fewer products: warp 0 also
-            // issues the update), warps 4-7 tokens 8..15 of the same columns (the same TMEM lanes)
+            // its hi / lo parts in TMEM; the four warps of a column take tokens 0..7, 8..10, 11..13
+            // and 14..15: 36, 30, 39 and 31 multiply-adds
+            constexpr int kFirst[5] = {0, 8, 11, 14, 16};
             float wq[L], cq[L], u[L], ul[L];
             tc::tmem_ld2x16(tl + G::kDW + L, tl + G::kDWc + L, wq, cq);
             tc::tmem_ld2x16(tl + G::kUHi, tl + G::kULo, u, ul);
@@ -541,7 +558,8 @@ __device__ __forceinline__ void chunk_interval(const StepParams& p, Stage& S, fl
             for (int t = 0; t < L; ++t) u[t] = __fadd_rn(u[t], ul[t]);
 #pragma unroll
             for (int t = 0; t < L; ++t) {
-                if ((t >= L / 2) != (hf == 1)) continue;
+                const int of = t >= kFirst[3] ? 3 : t >= kFirst[2] ? 2 : t >= kFirst[1] ? 1 : 0;
+                if (of != hf) continue;
                 float oa = __fadd_rn(wq[t], cq[t]), ob = 0.0f;
                 // row t of M, four entries per load
 #pragma unroll
@@ -559,7 +577,7 @@ __device__ __forceinline__ void chunk_interval(const StepParams& p, Stage& S, fl
         // S_e = fma(S_b, Dc_{L-1}, update): to TMEM (with its lo) for the next block, or, after
         // the interval's last block, to the row-major buffer
 #pragma unroll 1
-        for (int c0 = 64 * hf; c0 < 64 * hf + 64; c0 += 16) {
+        for (int c0 = 32 * hf; c0 < 32 * hf + 32; c0 += 16) {
             float x[16], up[16], lo[16];
             tc::tmem_ld2x16(tl + G::kHi + c0, tl + G::kUpd + c0, x, up);
 #pragma unroll
@@ -579,7 +597,7 @@ __device__ __forceinline__ void chunk_interval(const StepParams& p, Stage& S, fl
     if (p.t_begin >= p.t_end) {
         // no tokens: the state goes back unchanged
 #pragma unroll 1
-        for (int i0 = 64 * hf; i0 < 64 * hf + 64; i0 += 16) {
+        for (int i0 = 32 * hf; i0 < 32 * hf + 32; i0 += 16) {
             float x[16];
             tc::tmem_ld16(tl + G::kHi + i0, x);
 #pragma unroll

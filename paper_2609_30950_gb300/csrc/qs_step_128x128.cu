@@ -11,6 +11,6 @@ cudaError_t launch_wb_row_128x128(const qstate_cfg& cfg, const StepParams& p, cu
     return launch_wb_row_t<128, 128, 8>(cfg, p, stream);
 }
 cudaError_t launch_wb_chunk_128x128(const qstate_cfg& cfg, const StepParams& p, cudaStream_t stream) {
-    return launch_wb_row_t<128, 128, 8, true>(cfg, p, stream);
+    return launch_wb_row_t<128, 128, 16, true>(cfg, p, stream);
 }
 }  // namespace qs

@@ -73,13 +73,15 @@ struct WbGeom {
     static constexpr int RPB = RowQuant<DV>::RPB;   // row layout: rows per warp
 };
 
-template <int DK, int DV, int NW>
+template <int DK, int DV, int NW, bool CHUNK>
 struct alignas(16) WbSmem {
+    // the chunked form needs no partials, and its candidate tables lie in its operand tiles
+    static constexpr int NWP = CHUNK ? 0 : NW;
     WbStage<DK, DV> st[2];
     float sbuf[DK * DV];                  // FP32 state of the head (swizzled rows)
     union {
-        float red[2][NW][DV];             // p and r partials per warp (token phase)
-        float4 cand[NW][RowQuant<DV>::RPB][RowQuant<DV>::kTable];   // per warp and row: the candidates (fit_rows)
+        float red[2][NWP ? NWP : 1][NWP ? DV : 1];             // p and r partials per warp (token phase)
+        float4 cand[NWP ? NWP : 1][RowQuant<DV>::RPB][NWP ? RowQuant<DV>::kTable : 1];   // per warp and row: the candidates (fit_rows)
         int hist[17 * kNFit + 16];        // prep: counting sort of the rows (width, factor)
     } rc;
     float4 deqAS[DK];                     // (-A, -A, S, S) and (B, B): x = (2^23 + u - A) S + B,
@@ -247,8 +249,8 @@ __global__ void __launch_bounds__(NW * 32, CHUNK ? 1 : 2) wb_row_kernel(const Wb
     constexpr int RPW = Geo::RPW, CPL = Geo::CPL, CP2 = CPL / 2;
     constexpr int TPR = Geo::TPR, RPB = Geo::RPB, NB = DK / RPB;
     static_assert(CPL == 2 || CPL == 4, "value columns");
-    static_assert(RPW >= 2 && RPW <= 16 && NW == 8, "warps");
-    using Sm = WbSmem<DK, DV, NW>;
+    static_assert(RPW >= 2 && RPW <= 16 && NW == (CHUNK ? 16 : 8), "warps");
+    using Sm = WbSmem<DK, DV, NW, CHUNK>;
     using Stage = WbStage<DK, DV>;
     const StepParams& p = wp.s;
     extern __shared__ __align__(16) uint8_t smem_raw[];
@@ -658,6 +660,9 @@ __global__ void __launch_bounds__(NW * 32, CHUNK ? 1 : 2) wb_row_kernel(const Wb
 
         // ---- write-back (row layout) ----------------------------------------------------------
         const bool refit = (p.fit_every <= 1) || ((p.w_index + h) % p.fit_every == 0);
+        float4* cand;
+        if constexpr (CHUNK) cand = reinterpret_cast<float4*>(cb) + (warp * RPB + lane / TPR) * RowQuant<DV>::kTable;
+        else cand = sm.rc.cand[warp][lane / TPR];
         // Row batches are claimed dynamically (longest first, by the order above): the
         // search length varies with the width and the data.
         auto next_batch = [&]() {
@@ -704,7 +709,7 @@ __global__ void __launch_bounds__(NW * 32, CHUNK ? 1 : 2) wb_row_kernel(const Wb
             }
             const float4 wc = sm.wc[w > 16 ? 0 : w];
             if (refit) {
-                const int bk = fit_rows<DV>(av, m4, R, w, wc, sm.fitf, sm.rc.cand[warp][lane / TPR], lane, D);
+                const int bk = fit_rows<DV>(av, m4, R, w, wc, sm.fitf, cand, lane, D);
                 if (w >= 2) fidx = bk;
             } else if (w >= 2 && R > 0.0f) {
                 D = cand_step(sm.fitf[fidx], R, wc.y);
@@ -744,7 +749,7 @@ cudaError_t launch_wb_row_t(const qstate_cfg& cfg, const StepParams& sp, cudaStr
     wp.s.stage_bytes = DK * DV * cfg.bmax / 8;
     wp.nheads = cfg.B * cfg.H;
     const int pstride = (wp.s.stage_bytes + 32 + 15) & ~15;
-    const size_t smem = sizeof(WbSmem<DK, DV, NW>) + static_cast<size_t>(pstride) + (CHUNK ? ChunkGeo::kBytes : 0u);
+    const size_t smem = sizeof(WbSmem<DK, DV, NW, CHUNK>) + static_cast<size_t>(pstride) + (CHUNK ? ChunkGeo::kBytes : 0u);
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          static_cast<int>(smem));
     if (e != cudaSuccess) return e;
