@@ -205,6 +205,7 @@ __device__ __forceinline__ void chunk_interval(const StepParams& p, Stage& S, fl
         const int nb = min(L, p.t_end - tb);
         if (p.erase && tt < nb)
             cp_async4(stg + G::sB + (((tb - p.t_begin) / L) % 3) * L * 4 + tt * 4, p.beta + (tokb + tb + tt) * p.H + h);
+#pragma unroll 1
         for (int c = tt; c < nb * (D / 4); c += 128) {
             const int tau = c / (D / 4), part = c % (D / 4);
             const size_t tok = (tokb + tb + tau) * p.H + h;
@@ -213,6 +214,7 @@ __device__ __forceinline__ void chunk_interval(const StepParams& p, Stage& S, fl
             if (p.decay_row && !p.s_code) cp_async16(stg + G::sS + tau * D * 4 + part * 16, p.s + tok * D + part * 4);
         }
         if (p.decay_row && p.s_code) {
+#pragma unroll 1
             for (int c = tt; c < nb * (D / 16); c += 128) {
                 const int tau = c / (D / 16), part = c % (D / 16);
                 const size_t tok = (tokb + tb + tau) * p.H + h;
@@ -232,6 +234,7 @@ __device__ __forceinline__ void chunk_interval(const StepParams& p, Stage& S, fl
     // the last block's way out (global loads in flight would hold up every barrier)
     auto issue_v = [&](int tb) {
         const int nb = min(L, p.t_end - tb);
+#pragma unroll 1
         for (int c = tt; c < nb * (D / 4); c += 128) {
             const int tau = c / (D / 4), part = c % (D / 4);
             cp_async16(sbuf + tau * D + part * 4, p.v + ((tokb + tb + tau) * p.H + h) * D + part * 4);
@@ -450,7 +453,7 @@ __device__ __forceinline__ void chunk_interval(const StepParams& p, Stage& S, fl
             constexpr uint64_t kStepW = (2 * G::kLboW) >> 4, kStepH = (2 * G::kLboH) >> 4;
             uint64_t bh = tc::smem_desc(tc::smem_addr(bw_hi), G::kLboW, G::kSboW);
             if (tid == 0) {
-#pragma unroll
+#pragma unroll 4
                 for (int ks = 0; ks < D / 8; ++ks) {
                     const uint32_t acc = ks > 0 ? 1u : 0u;
                     tc::mma_tf32_ts(tmem + G::kDW, tmem + G::kHi + 8 * ks, bh, idW2, acc);
@@ -460,7 +463,7 @@ __device__ __forceinline__ void chunk_interval(const StepParams& p, Stage& S, fl
             } else {
                 uint64_t ah = tc::smem_desc(tc::smem_addr(kh_hi), G::kLboH, G::kSboH);
                 uint64_t al = tc::smem_desc(tc::smem_addr(kh_lo), G::kLboH, G::kSboH);
-#pragma unroll
+#pragma unroll 4
                 for (int ks = 0; ks < D / 8; ++ks) {
                     const uint32_t acc = ks > 0 ? 1u : 0u;
                     tc::mma_tf32_ss(tmem + G::kAM, ah, bh, idAM2, acc);
@@ -548,30 +551,46 @@ __device__ __forceinline__ void chunk_interval(const StepParams& p, Stage& S, fl
         }
         {
             // readouts of column j: o_t = (S_b^T (q o Dc))_t + sum_{s<=t} M_ts u_s, with u from
-            // its hi / lo parts in TMEM; the four warps of a column take tokens 0..7, 8..10, 11..13
-            // and 14..15: 36, 30, 39 and 31 multiply-adds
-            constexpr int kFirst[5] = {0, 8, 11, 14, 16};
-            float wq[L], cq[L], u[L], ul[L];
-            tc::tmem_ld2x16(tl + G::kDW + L, tl + G::kDWc + L, wq, cq);
+            // its hi / lo parts in TMEM.  The four warps of a column take four tokens each
+            // (4 hf + m); the terms go by fours of s, whole below the diagonal and triangular on it,
+            // so that one piece of code serves all warps (unrolled per token it was 10 KB)
+            float wq[4], cq[4], u[L], ul[L];
+            tc::tmem_ld2x4(tl + G::kDW + L + 4 * hf, tl + G::kDWc + L + 4 * hf, wq, cq);
             tc::tmem_ld2x16(tl + G::kUHi, tl + G::kULo, u, ul);
 #pragma unroll
             for (int t = 0; t < L; ++t) u[t] = __fadd_rn(u[t], ul[t]);
+            float oa[4], ob[4];
 #pragma unroll
-            for (int t = 0; t < L; ++t) {
-                const int of = t >= kFirst[3] ? 3 : t >= kFirst[2] ? 2 : t >= kFirst[1] ? 1 : 0;
-                if (of != hf) continue;
-                float oa = __fadd_rn(wq[t], cq[t]), ob = 0.0f;
-                // row t of M, four entries per load
-#pragma unroll
-                for (int s4 = 0; s4 <= t; s4 += 4) {
-                    const float4 m4 = reinterpret_cast<const float4*>(amM + t * L)[s4 / 4];
-                    if (s4 <= t) oa = fmaf(m4.x, u[s4], oa);
-                    if (s4 + 1 <= t) ob = fmaf(m4.y, u[s4 + 1], ob);
-                    if (s4 + 2 <= t) oa = fmaf(m4.z, u[s4 + 2], oa);
-                    if (s4 + 3 <= t) ob = fmaf(m4.w, u[s4 + 3], ob);
-                }
-                if (t < n) p.o[((tokb + t0 + t) * p.H + h) * D + jl] = oa + ob;
+            for (int m = 0; m < 4; ++m) {
+                oa[m] = __fadd_rn(wq[m], cq[m]);
+                ob[m] = 0.0f;
             }
+            const float4* M4 = reinterpret_cast<const float4*>(amM + 4 * hf * L);
+#pragma unroll
+            for (int g = 0; g < L / 4; ++g) {
+                if (g < hf) {
+#pragma unroll
+                    for (int m = 0; m < 4; ++m) {
+                        const float4 m4 = M4[m * (L / 4) + g];
+                        oa[m] = fmaf(m4.x, u[4 * g], oa[m]);
+                        ob[m] = fmaf(m4.y, u[4 * g + 1], ob[m]);
+                        oa[m] = fmaf(m4.z, u[4 * g + 2], oa[m]);
+                        ob[m] = fmaf(m4.w, u[4 * g + 3], ob[m]);
+                    }
+                } else if (g == hf) {
+#pragma unroll
+                    for (int m = 0; m < 4; ++m) {
+                        const float4 m4 = M4[m * (L / 4) + g];
+                        oa[m] = fmaf(m4.x, u[4 * g], oa[m]);
+                        if (m >= 1) ob[m] = fmaf(m4.y, u[4 * g + 1], ob[m]);
+                        if (m >= 2) oa[m] = fmaf(m4.z, u[4 * g + 2], oa[m]);
+                        if (m >= 3) ob[m] = fmaf(m4.w, u[4 * g + 3], ob[m]);
+                    }
+                }
+            }
+#pragma unroll
+            for (int m = 0; m < 4; ++m)
+                if (4 * hf + m < n) p.o[((tokb + t0 + 4 * hf + m) * p.H + h) * D + jl] = oa[m] + ob[m];
         }
         wait_mma(1);
         // S_e = fma(S_b, Dc_{L-1}, update): to TMEM (with its lo) for the next block, or, after

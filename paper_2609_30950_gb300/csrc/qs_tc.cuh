@@ -84,6 +84,22 @@ __device__ __forceinline__ void tmem_ld2x16(uint32_t ta, uint32_t tb, float (&va
         vb[c] = __uint_as_float(r[16 + c]);
     }
 }
+// Two 4-column loads in flight, then one wait.
+__device__ __forceinline__ void tmem_ld2x4(uint32_t ta, uint32_t tb, float (&va)[4], float (&vb)[4]) {
+    uint32_t r[8];
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%8];\n"
+        "tcgen05.ld.sync.aligned.32x32b.x4.b32 {%4,%5,%6,%7}, [%9];\n"
+        "tcgen05.wait::ld.sync.aligned;\n"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+        : "r"(ta), "r"(tb)
+        : "memory");
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+        va[c] = __uint_as_float(r[c]);
+        vb[c] = __uint_as_float(r[4 + c]);
+    }
+}
 __device__ __forceinline__ void tmem_st16(uint32_t taddr, const float (&v)[16]) {
     asm volatile(
         "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16};\n" ::"r"(

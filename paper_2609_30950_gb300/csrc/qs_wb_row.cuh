@@ -169,6 +169,7 @@ __device__ __forceinline__ void wb_issue_meta(WbStage<DK, DV>& S, int g, int gne
     const size_t rb = static_cast<size_t>(g) * DK;
     // one array at a time, in 16-byte chunks
     auto seg = [&](void* dst, const void* src, int nchunks) {
+#pragma unroll 1
         for (int c = t; c < nchunks; c += nt)
             cp_async16(static_cast<uint8_t*>(dst) + 16 * c, static_cast<const uint8_t*>(src) + 16 * c);
     };
@@ -232,8 +233,10 @@ __device__ __forceinline__ void wb_issue_payload(const WbStage<DK, DV>& S, uint8
         const int nbytes = S.in_end - S.in_off;
         const uint8_t* src = p.in_payload + static_cast<size_t>(b) * p.region_bytes + S.in_off;
         if (DV == 128) {
+#pragma unroll 1
             for (int i = tid; i < nbytes / 16; i += blockDim.x) cp_async16(pay + 16 * i, src + 16 * i);
         } else {
+#pragma unroll 1
             for (int i = tid; i < nbytes / 8; i += blockDim.x) cp_async8(pay + 8 * i, src + 8 * i);
         }
     }
