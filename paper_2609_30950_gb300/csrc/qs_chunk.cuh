@@ -164,6 +164,49 @@ __device__ __forceinline__ void chunk_teardown(uint32_t tmem, uint8_t* cb, int* 
     }
 }
 
+// Staging of the block at token tb of head (b, h) by 128 threads (tt): k, q, the rates and beta; one
+// commit group.
+__device__ __forceinline__ void chunk_issue_kqs(const StepParams& p, uint8_t* cb, int tb, int b, int h, int tt) {
+    using G = ChunkGeo;
+    constexpr int L = G::L, D = G::D;
+    uint8_t* stg = cb + G::oStg;
+    const size_t tokb = static_cast<size_t>(b) * p.T;
+    const int nb = min(L, p.t_end - tb);
+    if (p.erase && tt < nb)
+        cp_async4(stg + G::sB + (((tb - p.t_begin) / L) % 3) * L * 4 + tt * 4, p.beta + (tokb + tb + tt) * p.H + h);
+#pragma unroll 1
+    for (int c = tt; c < nb * (D / 4); c += 128) {
+        const int tau = c / (D / 4), part = c % (D / 4);
+        const size_t tok = (tokb + tb + tau) * p.H + h;
+        cp_async16(stg + G::sK + tau * D * 4 + part * 16, p.k + tok * D + part * 4);
+        cp_async16(stg + G::sQ + tau * D * 4 + part * 16, p.q + tok * D + part * 4);
+        if (p.decay_row && !p.s_code) cp_async16(stg + G::sS + tau * D * 4 + part * 16, p.s + tok * D + part * 4);
+    }
+    if (p.decay_row && p.s_code) {
+#pragma unroll 1
+        for (int c = tt; c < nb * (D / 16); c += 128) {
+            const int tau = c / (D / 16), part = c % (D / 16);
+            const size_t tok = (tokb + tb + tau) * p.H + h;
+            cp_async16(stg + G::sS + tau * D + part * 16, p.s_code + tok * D + part * 16);
+        }
+    } else if (!p.decay_row && tt < nb) {
+        const size_t tok = (tokb + tb + tt) * p.H + h;
+        if (p.s_code)   // one code per head and token: its level, stored directly
+            reinterpret_cast<float*>(stg + G::sS)[tt] =
+                __ldg(p.s_lut + static_cast<size_t>(h) * p.L + min(static_cast<int>(p.s_code[tok]), p.L - 1));
+        else
+            cp_async4(stg + G::sS + tt * 4, p.s + tok);
+    }
+    cp_async_commit();
+}
+
+// At the start of a head, by warps 8-11 (which have no part in its preparation): the first block's
+// inputs, which then arrive while the state is unpacked.
+__device__ __forceinline__ void chunk_prefetch(const StepParams& p, uint8_t* cb, int b, int h) {
+    const int tt = static_cast<int>(threadIdx.x) - 256;
+    if (tt >= 0 && tt < 128 && p.t_begin < p.t_end) chunk_issue_kqs(p, cb, p.t_begin, b, h, tt);
+}
+
 // The interval [p.t_begin, p.t_end) of head (b, h): the state arrives in sbuf (row-major,
 // swizzled) and leaves there; readouts go to p.o, the EMA statistics of the rows to S.ms / S.mr.
 // `phase` tracks the mbarriers' parities (uniform over the CTA).
@@ -200,36 +243,7 @@ __device__ __forceinline__ void chunk_interval(const StepParams& p, Stage& S, fl
         phase ^= 1u << which;
         tc::fence_after_sync();
     };
-    // staging of the block at token tb by the value-column threads: k, q, the rates and beta
-    auto issue_kqs = [&](int tb) {
-        const int nb = min(L, p.t_end - tb);
-        if (p.erase && tt < nb)
-            cp_async4(stg + G::sB + (((tb - p.t_begin) / L) % 3) * L * 4 + tt * 4, p.beta + (tokb + tb + tt) * p.H + h);
-#pragma unroll 1
-        for (int c = tt; c < nb * (D / 4); c += 128) {
-            const int tau = c / (D / 4), part = c % (D / 4);
-            const size_t tok = (tokb + tb + tau) * p.H + h;
-            cp_async16(stg + G::sK + tau * D * 4 + part * 16, p.k + tok * D + part * 4);
-            cp_async16(stg + G::sQ + tau * D * 4 + part * 16, p.q + tok * D + part * 4);
-            if (p.decay_row && !p.s_code) cp_async16(stg + G::sS + tau * D * 4 + part * 16, p.s + tok * D + part * 4);
-        }
-        if (p.decay_row && p.s_code) {
-#pragma unroll 1
-            for (int c = tt; c < nb * (D / 16); c += 128) {
-                const int tau = c / (D / 16), part = c % (D / 16);
-                const size_t tok = (tokb + tb + tau) * p.H + h;
-                cp_async16(stg + G::sS + tau * D + part * 16, p.s_code + tok * D + part * 16);
-            }
-        } else if (!p.decay_row && tt < nb) {
-            const size_t tok = (tokb + tb + tt) * p.H + h;
-            if (p.s_code)   // one code per head and token: its level, stored directly
-                reinterpret_cast<float*>(stg + G::sS)[tt] =
-                    __ldg(p.s_lut + static_cast<size_t>(h) * p.L + min(static_cast<int>(p.s_code[tok]), p.L - 1));
-            else
-                cp_async4(stg + G::sS + tt * 4, p.s + tok);
-        }
-        cp_async_commit();
-    };
+    auto issue_kqs = [&](int tb) { chunk_issue_kqs(p, cb, tb, b, h, tt); };
     // ... and v, into the row-major state buffer, which is free between the state's way in and
     // the last block's way out (global loads in flight would hold up every barrier)
     auto issue_v = [&](int tb) {
@@ -241,8 +255,6 @@ __device__ __forceinline__ void chunk_interval(const StepParams& p, Stage& S, fl
         }
         cp_async_commit();
     };
-    if (tt >= 0 && p.t_begin < p.t_end) issue_kqs(p.t_begin);
-
     // state in: S^T into TMEM (FP32 and lo); this thread's lane j, key rows of its half
 #pragma unroll 1
     for (int i0 = 32 * hf; i0 < 32 * hf + 32; i0 += 16) {
@@ -417,7 +429,7 @@ __device__ __forceinline__ void chunk_interval(const StepParams& p, Stage& S, fl
 
     RowA ra;   // phase A of the block about to start
     if (p.t_begin < p.t_end) {
-        if (tt >= 0) cp_async_wait_all();
+        cp_async_wait_all();                  // issued by chunk_prefetch's threads
         __syncthreads();                      // the first block's inputs; the state buffer is read
         if (tt >= 0) issue_v(p.t_begin);
         phase_a(p.t_begin, ra);
@@ -530,8 +542,6 @@ __device__ __forceinline__ void chunk_interval(const StepParams& p, Stage& S, fl
         }
         tc::fence_before_sync();
         __syncthreads();                                                            // C3
-        if (tt >= 0 && !last) issue_v(t0 + L);   // the solve is done with this block's v
-
         // update = u^T (k o Dc_{L-1} / Dc) on the tensor cores (3xTF32, K = 16 tokens)
         if (tid == 0) {
             tc::fence_after_sync();
@@ -549,6 +559,7 @@ __device__ __forceinline__ void chunk_interval(const StepParams& p, Stage& S, fl
             }
             tc::mma_commit(bar + 1);
         }
+        if (tt >= 0 && !last) issue_v(t0 + L);   // the solve is done with this block's v
         {
             // readouts of column j: o_t = (S_b^T (q o Dc))_t + sum_{s<=t} M_ts u_s, with u from
             // its hi / lo parts in TMEM.  The four warps of a column take four tokens each

@@ -297,6 +297,8 @@ __global__ void __launch_bounds__(NW * 32, CHUNK ? 1 : 2) wb_row_kernel(const Wb
             wb_issue_meta<DK, DV>(sm.st[sidx ^ 1], g + 1, g + 2 < g_end ? g + 2 : -1, S.nxt_in_off,
                                   S.nxt_in_end, S.nxt_out_off, wp, lane, 32);
 
+        if constexpr (CHUNK) chunk_prefetch(p, cb, b, h);
+
         // ---- prep ---------------------------------------------------------------------------
         const size_t tok0 = (static_cast<size_t>(b) * T + p.t_begin) * p.H + h;
         const float beta0 = p.erase ? S.beta : 1.0f;
