@@ -271,7 +271,8 @@ __device__ __forceinline__ void chunk_interval(const StepParams& p, Stage& S, fl
     tc::fence_before_sync();
 
     // Rows: thread (i, quarter qt) takes tokens 4 qt .. 4 qt + 3 of key row i.  Phase A (staged
-    // loads, decays, EMA terms) of block c + 1 runs while the tensor cores work on block c, the EMA
+    // loads, decays, EMA terms) of block c + 1 runs while the tensor cores work on block c (the two
+    // issuing warps, which stall on the product queue, run theirs beside the solve), the EMA
     // recursion over the first half's tokens beside the solve, and phase B (the second half's EMA
     // recursion, cumulative decays, operand tiles) at the start of block c + 1.  The quarters
     // exchange their decay products through shared memory; quarters 1 and 3 (warps 0-3 and 12-15,
@@ -487,10 +488,10 @@ __device__ __forceinline__ void chunk_interval(const StepParams& p, Stage& S, fl
             }
             tc::mma_commit(bar);
         }
-        // while the tensor cores work: phase A of the next block
-        if (!last) phase_a(t0 + L, ra);
+        // while the tensor cores work: phase A of the next block (by the issuing warps beside the solve)
+        if (!last && warp >= 2) phase_a(t0 + L, ra);
         wait_mma(0);
-        if (warp == 0) {
+        if (warp == 8) {
             // A and M to shared memory (lane s < L holds row s of the product): the hi*hi
             // accumulator plus the corrections' (one FP32 rounding)
             float x[L], y[L], xc[L], yc[L];
@@ -505,9 +506,7 @@ __device__ __forceinline__ void chunk_interval(const StepParams& p, Stage& S, fl
             }
         }
         __syncthreads();                                                            // C2
-        // every thread is done with the next block's staged inputs: the one after it
-        if (tt >= 0 && t0 + 2 * L < p.t_end) issue_kqs(t0 + 2 * L);
-
+        if (!last && warp < 2) phase_a(t0 + L, ra);
         if (!last) first_half(t0 + L, ra);
         if (hf == 1) {
             // u of column j, token by token: u_t = w_t v_t - (S_b^T (a o Dc))_t - sum_{s<t} A_ts u_s
@@ -559,7 +558,11 @@ __device__ __forceinline__ void chunk_interval(const StepParams& p, Stage& S, fl
             }
             tc::mma_commit(bar + 1);
         }
-        if (tt >= 0 && !last) issue_v(t0 + L);   // the solve is done with this block's v
+        if (tt >= 0 && !last) {
+            issue_v(t0 + L);   // the solve is done with this block's v
+            // every thread is done with the next block's staged inputs: the one after it
+            if (t0 + 2 * L < p.t_end) issue_kqs(t0 + 2 * L);
+        }
         {
             // readouts of column j: o_t = (S_b^T (q o Dc))_t + sum_{s<=t} M_ts u_s, with u from
             // its hi / lo parts in TMEM.  The four warps of a column take four tokens each
