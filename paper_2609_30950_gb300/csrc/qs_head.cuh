@@ -602,13 +602,17 @@ __device__ __forceinline__ void head_issue(HeadStage<DK, DV>& S, uint8_t* pay, c
         const int nbytes = DK * DV / 8 * m.w_in;
         const uint8_t* src = p.in_payload + static_cast<size_t>(b) * p.region_bytes + m.in_off;
         if (DV == 128) {
+#pragma unroll 1
             for (int i = tid; i < nbytes / 16; i += G::NT) hd_cp16(pay + 16 * i, src + 16 * i);
         } else {
+#pragma unroll 1
             for (int i = tid; i < nbytes / 8; i += G::NT) hd_cp8(pay + 8 * i, src + 8 * i);
         }
         const uint8_t* sc = reinterpret_cast<const uint8_t*>(p.in_scales + static_cast<size_t>(bh) * G::NSG);
+#pragma unroll 1
         for (int i = tid; i < G::NSG * 2 / 16; i += G::NT) hd_cp16(reinterpret_cast<uint8_t*>(S.sc) + 16 * i, sc + 16 * i);
         const uint8_t* fi = p.in_fidx + static_cast<size_t>(bh) * G::NSG;
+#pragma unroll 1
         for (int i = tid; i < G::NSG / 16; i += G::NT) hd_cp16(S.fidx + 16 * i, fi + 16 * i);
         if (p.t_end > p.t_begin) {
             const int h = bh - b * p.H;
@@ -717,6 +721,7 @@ __global__ void __launch_bounds__(HeadGeom<DK, DV>::NT, 2) head_wb_kernel(const 
         // zero the output rows: codes are OR-ed in
         {
             const int nz = (bytes_out + 16) / 16;
+#pragma unroll 1
             for (int i = tid; i < nz; i += NT) reinterpret_cast<uint4*>(pout)[i] = make_uint4(0, 0, 0, 0);
         }
         __syncthreads();                     // tail word written; stage scalars visible
@@ -870,13 +875,14 @@ __global__ void __launch_bounds__(HeadGeom<DK, DV>::NT, 2) head_wb_kernel(const 
             const bool refit = (p.fit_every <= 1) || ((p.w_index + h) % p.fit_every == 0);
             V Rg = hv_bc<V>(0.0f), Mg = hv_bc<V>(0.0f);
 #pragma unroll
-            for (int r = 0; r < 32; ++r) {
+            for (int r = 0; r < 32; ++r)
 #pragma unroll
-                for (int c = 0; c < CPL; ++c) {
-                    const float av = fabsf(hv_get(x[r], c));
-                    hv_set(Rg, c, fmaxf(hv_get(Rg, c), av));
-                    if (w == 1) hv_set(Mg, c, __fadd_rn(hv_get(Mg, c), av));   // in row order
-                }
+                for (int c = 0; c < CPL; ++c) hv_set(Rg, c, fmaxf(hv_get(Rg, c), fabsf(hv_get(x[r], c))));
+            if (w == 1) {   // the mean |x|, summed in row order
+#pragma unroll
+                for (int r = 0; r < 32; ++r)
+#pragma unroll
+                    for (int c = 0; c < CPL; ++c) hv_set(Mg, c, __fadd_rn(hv_get(Mg, c), fabsf(hv_get(x[r], c))));
             }
             int fidx[CPL];
             float D[CPL];
@@ -977,6 +983,7 @@ __global__ void __launch_bounds__(HeadGeom<DK, DV>::NT, 2) head_wb_kernel(const 
             __syncthreads();
             Vec* dst = reinterpret_cast<Vec*>(p.out_payload + static_cast<size_t>(b) * p.region_bytes + S.out_off);
             const Vec* srcv = reinterpret_cast<const Vec*>(pout);
+#pragma unroll 1
             for (int i = tid; i < bytes_out / static_cast<int>(sizeof(Vec)); i += NT) dst[i] = srcv[i];
         }
         if (stats && tid == DV) {
