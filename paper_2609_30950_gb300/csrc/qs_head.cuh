@@ -504,7 +504,7 @@ __device__ __forceinline__ void head_unpack_rows(const uint8_t* pay, int r0, int
 // (one width per head, so the kernel switches once per head): the lane's CPL codes of row r
 // (offset binary for W >= 2; for W = 1 the sign bit, 1 for x < 0, negative zero counting as
 // positive) are OR-ed into the row's bit stream at bit col0 W.  A lane's CPL W bits stay within
-// one word when CPL W divides 32; at CPL W = 32 the word is the lane's alone.
+// one word when CPL W divides 32; at CPL W = 8, 16 and 32 its bytes are the lane's alone.
 template <int W, int DV, int CPL, class V>
 __device__ __forceinline__ void head_pack_rows(const V (&x)[32], V inv2, uint8_t* pout, int r0, int col0) {
     constexpr int rowbytes = W * (DV / 8);
@@ -527,6 +527,10 @@ __device__ __forceinline__ void head_pack_rows(const V (&x)[32], V inv2, uint8_t
         uint32_t* wd = reinterpret_cast<uint32_t*>(reinterpret_cast<uint8_t*>(words) + r * rowbytes);
         if constexpr (CPL * W == 32) {
             *wd = chunk;
+        } else if constexpr (CPL * W == 16) {   // the lane's own bytes: no other lane's bits beside them
+            *reinterpret_cast<uint16_t*>(pout + (r0 + r) * rowbytes + 2 * (col0 / CPL)) = static_cast<uint16_t>(chunk);
+        } else if constexpr (CPL * W == 8) {
+            pout[(r0 + r) * rowbytes + col0 / CPL] = static_cast<uint8_t>(chunk);
         } else if constexpr (32 % (CPL * W) == 0) {
             if (chunk) atomicOr(wd, chunk << sh);
         } else {
