@@ -490,7 +490,9 @@ __device__ __forceinline__ void head_unpack_rows(const uint8_t* pay, int r0, int
         for (int r = 0; r < 32; ++r) {
             const uint32_t* wd = reinterpret_cast<const uint32_t*>(base + r * rowbytes);
             uint32_t chunk;
-            if constexpr (32 % (CPL * W) == 0) chunk = wd[0] >> sh;
+            if constexpr (CPL * W == 8) chunk = pay[(r0 + r) * rowbytes + col0 / CPL];   // the lane's own byte
+            else if constexpr (CPL * W == 16) chunk = reinterpret_cast<const uint16_t*>(pay)[((r0 + r) * rowbytes) / 2 + col0 / CPL];
+            else if constexpr (32 % (CPL * W) == 0) chunk = wd[0] >> sh;
             else chunk = __funnelshift_r(wd[0], wd[1], sh);
             V t;
 #pragma unroll
