@@ -193,7 +193,7 @@ __device__ __forceinline__ void chunk_issue_kqs(const StepParams& p, uint8_t* cb
         const size_t tok = (tokb + tb + tt) * p.H + h;
         if (p.s_code)   // one code per head and token: its level, stored directly
             reinterpret_cast<float*>(stg + G::sS)[tt] =
-                __ldg(p.s_lut + static_cast<size_t>(h) * p.L + min(static_cast<int>(p.s_code[tok]), p.L - 1));
+                *(p.s_lut + static_cast<size_t>(h) * p.L + min(static_cast<int>(p.s_code[tok]), p.L - 1));
         else
             cp_async4(stg + G::sS + tt * 4, p.s + tok);
     }
@@ -301,7 +301,7 @@ __device__ __forceinline__ void chunk_interval(const StepParams& p, Stage& S, fl
             } else if (p.s_code) {
                 const int code = min(static_cast<int>(sc[tau * D + i]), p.L - 1);
                 rate = p.L <= 4 ? S.lut[i * p.L + code]
-                                : __ldg(p.s_lut + (static_cast<size_t>(h) * D + i) * p.L + code);
+                                : *(p.s_lut + (static_cast<size_t>(h) * D + i) * p.L + code);
             } else {
                 rate = ss[tau * D + i];
             }

@@ -21,7 +21,8 @@ constexpr uint32_t kMagicBits = 0x4B400000u;
 constexpr uint32_t kTwo23Bits = 0x4B000000u;
 
 // Start of a kernel launched by launch_chained: waits until the launches before it in the stream are
-// complete and their writes visible (nothing global is touched before), then lets the one after
+// complete and their writes visible (nothing global is touched before, and nothing after through
+// the read-only path, whose data must not change while a kernel runs), then lets the one after
 // it take its place on idle SMs.
 __device__ __forceinline__ void chain_wait() {
     asm volatile("griddepcontrol.wait;" ::: "memory");

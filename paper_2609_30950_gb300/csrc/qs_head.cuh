@@ -582,13 +582,14 @@ __device__ __forceinline__ void hd_wait_all() { asm volatile("cp.async.wait_grou
 struct HeadMeta {
     int w_in, w_out, in_off, out_off, ok;
 };
-// (loads and check apart, so that a caller's other loads can be in flight with these)
+// (loads and check apart, so that a caller's other loads can be in flight with these; plain loads: the
+// launch before, which may still run when this one starts, writes what they read)
 __device__ __forceinline__ HeadMeta head_meta_load(const StepParams& p, int bh) {
     HeadMeta m;
-    m.w_in = __ldg(p.in_widths + bh);
-    m.w_out = __ldg(p.out_widths + bh);
-    m.in_off = static_cast<int>(__ldg(p.in_head_off + bh));
-    m.out_off = static_cast<int>(__ldg(p.out_head_off + bh));
+    m.w_in = *(p.in_widths + bh);
+    m.w_out = *(p.out_widths + bh);
+    m.in_off = static_cast<int>(*(p.in_head_off + bh));
+    m.out_off = static_cast<int>(*(p.out_head_off + bh));
     m.ok = 0;
     return m;
 }
@@ -686,19 +687,19 @@ __global__ void __launch_bounds__(HeadGeom<DK, DV>::NT, 2) head_wb_kernel(const 
         if (tid == 0) {
             if (g_begin + 1 < g_end) l1 = head_meta_load(p, g_begin + 1);
             if (has_tokens) {
-                if (p.erase) beta = __ldg(p.beta + tok);
+                if (p.erase) beta = *(p.beta + tok);
                 if (p.s_code) code = p.s_code[tok];
-                else rate = __ldg(p.s + tok);
+                else rate = *(p.s + tok);
             }
             if (stats) {
-                ms = __ldg(p.ema_s + g_begin);
-                mr = __ldg(p.ema_r + g_begin);
+                ms = *(p.ema_s + g_begin);
+                mr = *(p.ema_r + g_begin);
             }
         }
         const HeadMeta m0 = head_meta_check<DK, DV>(p, l0);
         head_issue<DK, DV>(S, pin0, m0, g_begin, p);
         if (tid == 0) {
-            if (has_tokens && p.s_code) rate = __ldg(p.s_lut + static_cast<size_t>(h) * p.L + min(code, p.L - 1));
+            if (has_tokens && p.s_code) rate = *(p.s_lut + static_cast<size_t>(h) * p.L + min(code, p.L - 1));
             S.w_in = m0.w_in; S.w_out = m0.w_out; S.in_off = m0.in_off; S.out_off = m0.out_off; S.ok = m0.ok;
             S.beta = beta; S.rate = rate; S.ms = ms; S.mr = mr;
             nmeta = head_meta_check<DK, DV>(p, l1);
@@ -721,12 +722,12 @@ __global__ void __launch_bounds__(HeadGeom<DK, DV>::NT, 2) head_wb_kernel(const 
                 // the next head's scalars and the metadata after it: loads now, stored below
                 const int nb = (bh + 1) / p.H, nh = (bh + 1) - nb * p.H;
                 const size_t ntok = (static_cast<size_t>(nb) * p.T + p.t_begin) * p.H + nh;
-                nbeta = (has_tokens && p.erase) ? __ldg(p.beta + ntok) : 1.0f;
+                nbeta = (has_tokens && p.erase) ? *(p.beta + ntok) : 1.0f;
                 nrate = !has_tokens ? 1.0f
-                        : p.s_code ? __ldg(p.s_lut + static_cast<size_t>(nh) * p.L + min(static_cast<int>(p.s_code[ntok]), p.L - 1))
-                                   : __ldg(p.s + ntok);
-                nms = stats ? __ldg(p.ema_s + bh + 1) : 0.0f;
-                nmr = stats ? __ldg(p.ema_r + bh + 1) : 0.0f;
+                        : p.s_code ? *(p.s_lut + static_cast<size_t>(nh) * p.L + min(static_cast<int>(p.s_code[ntok]), p.L - 1))
+                                   : *(p.s + ntok);
+                nms = stats ? *(p.ema_s + bh + 1) : 0.0f;
+                nmr = stats ? *(p.ema_r + bh + 1) : 0.0f;
                 if (bh + 2 < g_end) m2 = head_meta<DK, DV>(p, bh + 2);
             }
         }
@@ -785,17 +786,17 @@ __global__ void __launch_bounds__(HeadGeom<DK, DV>::NT, 2) head_wb_kernel(const 
             const bool first = t == p.t_begin;
             if (!first) __syncthreads();     // every warp is done with the previous token's k, u
             const size_t tok = (static_cast<size_t>(b) * p.T + t) * p.H + h;
-            const float beta = first ? S.beta : (p.erase ? __ldg(p.beta + tok) : 1.0f);
+            const float beta = first ? S.beta : (p.erase ? *(p.beta + tok) : 1.0f);
             const float rate = first ? S.rate
-                                     : p.s_code ? __ldg(p.s_lut + static_cast<size_t>(h) * p.L +
+                                     : p.s_code ? *(p.s_lut + static_cast<size_t>(h) * p.L +
                                                         min(static_cast<int>(p.s_code[tok]), p.L - 1))
-                                                : __ldg(p.s + tok);
+                                                : *(p.s + tok);
             if (tid == 0 && (!(rate > 0.0f) || !(rate < INFINITY))) raise_status(p.status, QS_DEV_RATE);
             if (tid < DK) {
                 const int i = tid;
-                const float kk = first ? S.k[i] : __ldg(p.k + tok * DK + i);
-                const float qq = first ? S.q[i] : __ldg(p.q + tok * DK + i);
-                const float ai = p.general ? __ldg(p.a_in + tok * DK + i) : __fmul_rn(beta, kk);
+                const float kk = first ? S.k[i] : *(p.k + tok * DK + i);
+                const float qq = first ? S.q[i] : *(p.q + tok * DK + i);
+                const float ai = p.general ? *(p.a_in + tok * DK + i) : __fmul_rn(beta, kk);
                 sm.aq[i] = make_float4(ai, ai, qq, qq);
                 sm.kk[i] = make_float2(kk, kk);
                 const float kq = warp_sum(kk * qq);
@@ -813,8 +814,8 @@ __global__ void __launch_bounds__(HeadGeom<DK, DV>::NT, 2) head_wb_kernel(const 
                 }
             }
             if (tid < DV) {
-                sm.v[tid] = first ? S.v[tid] : __ldg(p.v + tok * DV + tid);
-                if (p.general) sm.gw[tid] = __ldg(p.w_in + tok * DV + tid);
+                sm.v[tid] = first ? S.v[tid] : *(p.v + tok * DV + tid);
+                if (p.general) sm.gw[tid] = *(p.w_in + tok * DV + tid);
             }
             __syncthreads();
             const V d2 = hv_bc<V>(expf(-rate));

@@ -304,7 +304,7 @@ __global__ void __launch_bounds__(NW * 32, CHUNK ? 1 : 2) wb_row_kernel(const Wb
         const float beta0 = p.erase ? S.beta : 1.0f;
         float rate_h = 0.0f;
         if (!p.decay_row)
-            rate_h = p.s_code ? __ldg(p.s_lut + static_cast<size_t>(h) * p.L +
+            rate_h = p.s_code ? *(p.s_lut + static_cast<size_t>(h) * p.L +
                                       min(static_cast<int>(p.s_code[tok0]), p.L - 1))
                               : S.rate_h;
         if (warp < 2) {
@@ -349,7 +349,7 @@ __global__ void __launch_bounds__(NW * 32, CHUNK ? 1 : 2) wb_row_kernel(const Wb
                 if (p.s_code) {
                     const int code = min(static_cast<int>(S.scode[i]), p.L - 1);
                     rate = p.L <= 4 ? S.lut[i * p.L + code]
-                                    : __ldg(p.s_lut + (static_cast<size_t>(h) * DK + i) * p.L + code);
+                                    : *(p.s_lut + (static_cast<size_t>(h) * DK + i) * p.L + code);
                 } else {
                     rate = S.s[i];
                 }
@@ -460,16 +460,16 @@ __global__ void __launch_bounds__(NW * 32, CHUNK ? 1 : 2) wb_row_kernel(const Wb
         float rk = 0.0f, rq = 0.0f, rs = 0.0f, rbeta = 1.0f, rv = 0.0f, ra = 0.0f, rw = 0.0f;
         int rc = 0;
         auto load_raw = [&](size_t tn) {
-            rk = __ldg(p.k + tn * DK + pi);
-            rq = __ldg(p.q + tn * DK + pi);
+            rk = *(p.k + tn * DK + pi);
+            rq = *(p.q + tn * DK + pi);
             const size_t si = p.decay_row ? tn * DK + pi : tn;
             if (p.s_code) rc = p.s_code[si];
-            else rs = __ldg(p.s + si);
-            if (p.erase) rbeta = __ldg(p.beta + tn);
-            if (p.general) ra = __ldg(p.a_in + tn * DK + pi);
+            else rs = *(p.s + si);
+            if (p.erase) rbeta = *(p.beta + tn);
+            if (p.general) ra = *(p.a_in + tn * DK + pi);
             if (prep_v) {
-                rv = __ldg(p.v + tn * DV + pi);
-                if (p.general) rw = __ldg(p.w_in + tn * DV + pi);
+                rv = *(p.v + tn * DV + pi);
+                if (p.general) rw = *(p.w_in + tn * DV + pi);
             }
         };
         if (!CHUNK && prep_k && p.t_begin + 1 < p.t_end) load_raw(tok0 + p.H);
@@ -582,9 +582,9 @@ __global__ void __launch_bounds__(NW * 32, CHUNK ? 1 : 2) wb_row_kernel(const Wb
                     const int code = min(rc, p.L - 1);
                     if (p.decay_row)
                         rate = p.L <= 4 ? S.lut[i * p.L + code]
-                                        : __ldg(p.s_lut + (static_cast<size_t>(h) * DK + i) * p.L + code);
+                                        : *(p.s_lut + (static_cast<size_t>(h) * DK + i) * p.L + code);
                     else
-                        rate = __ldg(p.s_lut + static_cast<size_t>(h) * p.L + code);
+                        rate = *(p.s_lut + static_cast<size_t>(h) * p.L + code);
                 } else {
                     rate = rs;
                 }
