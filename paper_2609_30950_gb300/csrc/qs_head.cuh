@@ -782,21 +782,37 @@ __global__ void __launch_bounds__(HeadGeom<DK, DV>::NT, 2) head_wb_kernel(const 
             sm.ms = S.ms;
             sm.mr = S.mr;
         }
+        // the inputs of token t + 1 are loaded into registers as soon as token t's are in shared memory
+        // (a token waited for its own loads before: 14 x 36 heads of 64 x 64, 275 tokens 1990 -> 699 us)
+        float nk = 0.0f, nq = 0.0f, na = 0.0f, nv = 0.0f, nw = 0.0f, tbeta = 1.0f, trate = 1.0f;
+        auto load_token = [&](int t) {
+            const size_t tok = (static_cast<size_t>(b) * p.T + t) * p.H + h;
+            if (tid < DK) {
+                nk = p.k[tok * DK + tid];
+                nq = p.q[tok * DK + tid];
+            }
+            if (tid < DV) nv = p.v[tok * DV + tid];
+            if (p.erase) tbeta = p.beta[tok];
+            trate = p.s_code ? p.s_lut[static_cast<size_t>(h) * p.L + min(static_cast<int>(p.s_code[tok]), p.L - 1)] : p.s[tok];
+        };
+        auto load_general = [&](int t) {
+            const size_t tok = (static_cast<size_t>(b) * p.T + t) * p.H + h;
+            if (tid < DK) na = p.a_in[tok * DK + tid];
+            if (tid < DV) nw = p.w_in[tok * DV + tid];
+        };
+        if (p.general) load_general(p.t_begin);
         for (int t = p.t_begin; t < p.t_end; ++t) {
             const bool first = t == p.t_begin;
             if (!first) __syncthreads();     // every warp is done with the previous token's k, u
             const size_t tok = (static_cast<size_t>(b) * p.T + t) * p.H + h;
-            const float beta = first ? S.beta : (p.erase ? *(p.beta + tok) : 1.0f);
-            const float rate = first ? S.rate
-                                     : p.s_code ? *(p.s_lut + static_cast<size_t>(h) * p.L +
-                                                        min(static_cast<int>(p.s_code[tok]), p.L - 1))
-                                                : *(p.s + tok);
+            const float beta = first ? S.beta : tbeta;
+            const float rate = first ? S.rate : trate;
             if (tid == 0 && (!(rate > 0.0f) || !(rate < INFINITY))) raise_status(p.status, QS_DEV_RATE);
             if (tid < DK) {
                 const int i = tid;
-                const float kk = first ? S.k[i] : *(p.k + tok * DK + i);
-                const float qq = first ? S.q[i] : *(p.q + tok * DK + i);
-                const float ai = p.general ? *(p.a_in + tok * DK + i) : __fmul_rn(beta, kk);
+                const float kk = first ? S.k[i] : nk;
+                const float qq = first ? S.q[i] : nq;
+                const float ai = p.general ? na : __fmul_rn(beta, kk);
                 sm.aq[i] = make_float4(ai, ai, qq, qq);
                 sm.kk[i] = make_float2(kk, kk);
                 const float kq = warp_sum(kk * qq);
@@ -814,8 +830,12 @@ __global__ void __launch_bounds__(HeadGeom<DK, DV>::NT, 2) head_wb_kernel(const 
                 }
             }
             if (tid < DV) {
-                sm.v[tid] = first ? S.v[tid] : *(p.v + tok * DV + tid);
-                if (p.general) sm.gw[tid] = *(p.w_in + tok * DV + tid);
+                sm.v[tid] = first ? S.v[tid] : nv;
+                if (p.general) sm.gw[tid] = nw;
+            }
+            if (t + 1 < p.t_end) {
+                load_token(t + 1);
+                if (p.general) load_general(t + 1);
             }
             __syncthreads();
             const V d2 = hv_bc<V>(expf(-rate));
