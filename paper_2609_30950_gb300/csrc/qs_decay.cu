@@ -34,12 +34,16 @@ __global__ void decay_init_kernel(float* lut, int nchan, int L) {
 
 // How a launch walks the rates 16 bytes at a time: LC lanes cover P = 4 LC consecutive values, a
 // chunk of one row's channels (P divides nchan) or several whole rows (nchan divides P), so a lane's
-// channels are fixed; 256 / LC such strips per block step through the strips of its chunk.
+// channels are fixed; 256 / LC such strips per block step through the strips of its chunk.  Other
+// channel counts up to kAnyChannels (ANY, one chunk) take a number of blocks for which the step is a
+// multiple of nchan: a lane's channels are fixed too, but differ between the strips of a block.
 struct Walk {
-    long long total, pitch;   // values in all; between a chunk's consecutive strips
+    long long total, pitch;   // values in whole groups of 4; between a chunk's consecutive strips
     long long strips;         // strips per chunk
     int chunks, nchan;
+    int tail;                 // values after the whole groups (0 to 3), by the first block's first threads
 };
+constexpr int kAnyChannels = 256;
 constexpr int kDecayThreads = 256, kInFlight = 4;
 // Blocks per SM, all resident, so that the sweeps keep their order: by the registers that the
 // thresholds take.
@@ -47,12 +51,13 @@ constexpr int kMinmaxBlocks = 5;
 constexpr uint32_t kMaxRate = 0x7f7fffffu;   // the largest finite float
 constexpr int codes_blocks(int lm1) { return lm1 <= 3 ? 5 : lm1 <= 7 ? 3 : 2; }
 
-template <int LC>
+template <int LC, bool ANY>
 __global__ void __launch_bounds__(kDecayThreads, kMinmaxBlocks) decay_minmax_rows_kernel(const float* __restrict__ s, const Walk wk, int L,
                                                                           float* lut, int* status) {
     constexpr int RS = kDecayThreads / LC;
     __shared__ uint4 smn[RS][LC], smx[RS][LC];
-    __shared__ uint32_t cmn[4 * LC], cmx[4 * LC];
+    constexpr int NC = ANY ? kAnyChannels : 4 * LC;
+    __shared__ uint32_t cmn[NC], cmx[NC];
     const int lane = threadIdx.x % LC, sub = threadIdx.x / LC;
     const int chunk = blockIdx.x % wk.chunks;
     const long long slices = gridDim.x / wk.chunks, step = slices * RS;
@@ -80,15 +85,15 @@ __global__ void __launch_bounds__(kDecayThreads, kMinmaxBlocks) decay_minmax_row
     }
     for (; m < mine; ++m) take(__ldg(reinterpret_cast<const uint4*>(at + m * d)));
     const bool bad = mine > 0 && (min(min(mn.x, mn.y), min(mn.z, mn.w)) < 1u || max(max(mx.x, mx.y), max(mx.z, mx.w)) > kMaxRate);
+    auto good = [](uint32_t v, uint32_t& lo, uint32_t& hi) {
+        if (v < 1u || v > kMaxRate) return false;
+        lo = min(lo, v);
+        hi = max(hi, v);
+        return true;
+    };
     if (bad) {
         // once more, the good rates only
         raise_status(status, QS_DEV_RATE);
-        auto good = [](uint32_t v, uint32_t& lo, uint32_t& hi) {
-            if (v >= 1u && v <= kMaxRate) {
-                lo = min(lo, v);
-                hi = max(hi, v);
-            }
-        };
         mn = make_uint4(~0u, ~0u, ~0u, ~0u);
         mx = make_uint4(0u, 0u, 0u, 0u);
 #pragma unroll 1
@@ -102,21 +107,44 @@ __global__ void __launch_bounds__(kDecayThreads, kMinmaxBlocks) decay_minmax_row
     }
     smn[sub][lane] = mn;
     smx[sub][lane] = mx;
-    for (int i = threadIdx.x; i < 4 * LC; i += kDecayThreads) {
+    for (int i = threadIdx.x; i < NC; i += kDecayThreads) {
         cmn[i] = kMaxRate + 1u;   // infinity
         cmx[i] = 0u;
     }
     __syncthreads();
-    // the strips' extrema of each of the P values, then of each channel among them
-    const int nc = min(wk.nchan, 4 * LC);
-    for (int i = threadIdx.x; i < 4 * LC; i += kDecayThreads) {
-        uint32_t lo = ~0u, hi = 0u;
-        for (int k = 0; k < RS; ++k) {
-            lo = min(lo, reinterpret_cast<const uint32_t*>(smn[k])[i]);
-            hi = max(hi, reinterpret_cast<const uint32_t*>(smx[k])[i]);
+    // the extrema of the block's 1024 values in turn, then of each channel among them
+    const uint32_t *vmn = reinterpret_cast<const uint32_t*>(smn), *vmx = reinterpret_cast<const uint32_t*>(smx);
+    const int nc = ANY ? wk.nchan : min(wk.nchan, 4 * LC);
+    if constexpr (ANY) {
+        // the block's values follow one another from a multiple of 1024 on: every nc-th is a channel's
+        const int per = kDecayThreads / nc, t = threadIdx.x;
+        if (t < per * nc) {
+            uint32_t lo = ~0u, hi = 0u;
+            for (int i = t; i < 4 * kDecayThreads; i += per * nc) {
+                lo = min(lo, vmn[i]);
+                hi = max(hi, vmx[i]);
+            }
+            const int ch = static_cast<int>((static_cast<long long>(blockIdx.x) * 4 * kDecayThreads + t) % nc);
+            atomicMin(&cmn[ch], lo);
+            atomicMax(&cmx[ch], hi);
         }
-        atomicMin(&cmn[i % nc], lo);
-        atomicMax(&cmx[i % nc], hi);
+    } else {
+        for (int i = threadIdx.x; i < 4 * LC; i += kDecayThreads) {
+            uint32_t lo = ~0u, hi = 0u;
+            for (int k = 0; k < RS; ++k) {
+                lo = min(lo, vmn[k * 4 * LC + i]);
+                hi = max(hi, vmx[k * 4 * LC + i]);
+            }
+            atomicMin(&cmn[i % nc], lo);
+            atomicMax(&cmx[i % nc], hi);
+        }
+    }
+    if (blockIdx.x == 0 && static_cast<int>(threadIdx.x) < wk.tail) {
+        const long long e = wk.total + threadIdx.x;
+        uint32_t lo = ~0u, hi = 0u;
+        if (!good(__ldg(reinterpret_cast<const uint32_t*>(s) + e), lo, hi)) raise_status(status, QS_DEV_RATE);
+        atomicMin(&cmn[e % nc], lo);
+        atomicMax(&cmx[e % nc], hi);
     }
     __syncthreads();
     for (int i = threadIdx.x; i < nc; i += kDecayThreads) {
@@ -126,7 +154,8 @@ __global__ void __launch_bounds__(kDecayThreads, kMinmaxBlocks) decay_minmax_row
     }
 }
 
-// Any channel count and alignment: thread e0 visits elements e0, e0 + S, e0 + 2S, ... with S a
+// Any channel count and alignment (unaligned rates; more than kAnyChannels channels that are no
+// multiple of 64): thread e0 visits elements e0, e0 + S, e0 + 2S, ... with S a
 // multiple of nchan, so its channel is fixed.
 __global__ void decay_minmax_kernel(const float* __restrict__ s, long long total, int nchan,
                                     int L, float* lut, int* status) {
@@ -186,7 +215,7 @@ __global__ void __launch_bounds__(kLevelThreads) decay_levels_kernel(float* lut,
 }
 
 // Codes from the last strip down.  LM1 thresholds for each of the lane's 4 channels in registers.
-template <int LC, int LM1>
+template <int LC, int LM1, bool ANY>
 __global__ void __launch_bounds__(kDecayThreads, codes_blocks(LM1)) decay_codes_rows_kernel(const float* __restrict__ s, const Walk wk,
                                                                          const float* __restrict__ thr,
                                                                          uint8_t* __restrict__ codes) {
@@ -195,16 +224,25 @@ __global__ void __launch_bounds__(kDecayThreads, codes_blocks(LM1)) decay_codes_
     const int chunk = blockIdx.x % wk.chunks;
     const long long slices = gridDim.x / wk.chunks, step = slices * RS;
     const long long off = static_cast<long long>(chunk) * 4 * LC + lane * 4;
+    const long long r0 = static_cast<long long>(blockIdx.x / wk.chunks) * RS + sub;   // strips from the end
     float th[4][LM1];
+    if (blockIdx.x == 0 && static_cast<int>(threadIdx.x) < wk.tail) {
+        const long long e = wk.total + threadIdx.x;
+        const float x = __ldg(s + e), *t = thr + static_cast<size_t>(e % wk.nchan) * LM1;
+        int c = 0;
+        for (int k = 0; k < LM1; ++k) c += x >= __ldg(t + k) ? 1 : 0;
+        codes[e] = static_cast<uint8_t>(c);
+    }
+    if (r0 >= wk.strips) return;
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
-        const size_t ch = static_cast<size_t>(chunk) * 4 * LC + (lane * 4 + j) % min(wk.nchan, 4 * LC);
+        const size_t ch = ANY ? static_cast<size_t>(((wk.strips - 1 - r0) * wk.pitch + off + j) % wk.nchan)
+                              : static_cast<size_t>(chunk) * 4 * LC + (lane * 4 + j) % min(wk.nchan, 4 * LC);
 #pragma unroll
         for (int k = 0; k < LM1; ++k) th[j][k] = __ldg(thr + ch * LM1 + k);
     }
-    const long long r0 = static_cast<long long>(blockIdx.x / wk.chunks) * RS + sub;   // strips from the end
     const long long d = step * wk.pitch;
-    long long left = r0 < wk.strips ? (wk.strips - 1 - r0) / step + 1 : 0;
+    long long left = (wk.strips - 1 - r0) / step + 1;
     long long e = (wk.strips - 1 - r0) * wk.pitch + off;
     if (left > 0 && e >= wk.total) {   // last strip of a short walk
         e -= d;
@@ -255,29 +293,41 @@ cudaError_t launch_quant_decay(const float* s, long long count, int nchan, int g
     const int L = 1 << g;
     const long long total = count * nchan;
     decay_init_kernel<<<(nchan + 255) / 256, 256, 0, stream>>>(lut, nchan, L);
-    // the 16-byte walk where a lane's channels can stay fixed: row decay always (channels a multiple
-    // of 64), heads when their number divides 128; up to 16 levels, whose thresholds fit in registers
+    // The 16-byte walk where a lane's channels can stay fixed: row decay always (channels a multiple
+    // of 64), heads up to kAnyChannels; codes of up to 16 levels, whose thresholds fit in registers.
+    // A rate at a time, every thread's extrema went to the few channels by global atomics: call by
+    // call from a cold L2, 118 x 256 x 12 rates took 221 us and 256 x 1024 x 1 took 360 us; the walk
+    // takes 30 and 28 us (of which 14 us are the call and its four launches).
     const bool aligned = (reinterpret_cast<uintptr_t>(s) & 15) == 0 && (reinterpret_cast<uintptr_t>(codes) & 3) == 0;
-    const int lc = nchan % 128 == 0 || (nchan % 4 == 0 && 128 % nchan == 0) ? 32 : nchan % 64 == 0 ? 16 : 0;
+    const bool fixed = nchan % 128 == 0 || 128 % nchan == 0;
+    const int lc = fixed || (nchan % 64 != 0 && nchan <= kAnyChannels) ? 32 : nchan % 64 == 0 ? 16 : 0;
+    const bool any = lc == 32 && !fixed;
     const bool walk = aligned && lc > 0;
     Walk wk = {};
+    long long turn = 1;   // blocks after which a strip meets the same channels again
     if (walk) {
         const int P = 4 * lc;
-        wk.total = total;
+        wk.tail = static_cast<int>(total & 3);
+        wk.total = total - wk.tail;
         wk.nchan = nchan;
-        wk.chunks = std::max(1, nchan / P);
-        wk.pitch = std::max(nchan, P);
-        wk.strips = (total + wk.pitch - 1) / wk.pitch;
+        wk.chunks = any ? 1 : std::max(1, nchan / P);
+        wk.pitch = any ? P : std::max(nchan, P);
+        wk.strips = (wk.total + wk.pitch - 1) / wk.pitch;
+        if (any) turn = nchan / gcd_ll(nchan, 4 * kDecayThreads);
     }
     // resident blocks, a whole number per chunk; fewer when there are not two strips for each lane
     auto blocks_of = [&](int per_sm) {
         const long long rs = kDecayThreads / lc;
         const long long want = std::max(1LL, static_cast<long long>(device_sm_count()) * per_sm / wk.chunks);
-        return static_cast<unsigned>(wk.chunks * std::max(1LL, std::min(want, (wk.strips + rs * 2 - 1) / (rs * 2))));
+        const long long b = std::max(1LL, std::min(want, (wk.strips + rs * 2 - 1) / (rs * 2)));
+        return static_cast<unsigned>(wk.chunks * (any ? std::max(turn, b / turn * turn) : b));
     };
     if (walk) {
-        if (lc == 32) decay_minmax_rows_kernel<32><<<blocks_of(kMinmaxBlocks), kDecayThreads, 0, stream>>>(s, wk, L, lut, status);
-        else decay_minmax_rows_kernel<16><<<blocks_of(kMinmaxBlocks), kDecayThreads, 0, stream>>>(s, wk, L, lut, status);
+#define QS_DM(LC, ANY) decay_minmax_rows_kernel<LC, ANY><<<blocks_of(kMinmaxBlocks), kDecayThreads, 0, stream>>>(s, wk, L, lut, status)
+        if (any) QS_DM(32, true);
+        else if (lc == 32) QS_DM(32, false);
+        else QS_DM(16, false);
+#undef QS_DM
     } else {
         // S = a multiple of lcm(nchan, 256) near (SMs x 8) CTAs of 256 threads
         const long long lcm = static_cast<long long>(nchan) / gcd_ll(nchan, 256) * 256;
@@ -290,18 +340,21 @@ cudaError_t launch_quant_decay(const float* s, long long count, int nchan, int g
     decay_levels_kernel<<<(nchan + per - 1) / per, kLevelThreads, 0, stream>>>(lut, thr, nchan, L, per, status);
     const unsigned blocks = static_cast<unsigned>(device_sm_count()) * 8u;
     if (walk && L <= 16) {
-#define QS_DC(LC, LM1) decay_codes_rows_kernel<LC, LM1><<<blocks_of(codes_blocks(LM1)), kDecayThreads, 0, stream>>>(s, wk, thr, codes)
-        if (lc == 32) {
-            if (L == 2) QS_DC(32, 1);
-            else if (L == 4) QS_DC(32, 3);
-            else if (L == 8) QS_DC(32, 7);
-            else QS_DC(32, 15);
+#define QS_DC(LC, LM1, ANY) \
+    decay_codes_rows_kernel<LC, LM1, ANY><<<blocks_of(codes_blocks(LM1)), kDecayThreads, 0, stream>>>(s, wk, thr, codes)
+#define QS_DL(LC, ANY)                     \
+    if (L == 2) QS_DC(LC, 1, ANY);         \
+    else if (L == 4) QS_DC(LC, 3, ANY);    \
+    else if (L == 8) QS_DC(LC, 7, ANY);    \
+    else QS_DC(LC, 15, ANY)
+        if (any) {
+            QS_DL(32, true);
+        } else if (lc == 32) {
+            QS_DL(32, false);
         } else {
-            if (L == 2) QS_DC(16, 1);
-            else if (L == 4) QS_DC(16, 3);
-            else if (L == 8) QS_DC(16, 7);
-            else QS_DC(16, 15);
+            QS_DL(16, false);
         }
+#undef QS_DL
 #undef QS_DC
     } else {
         decay_codes_generic_kernel<<<blocks, 256, 0, stream>>>(s, total, nchan, L - 1, thr, codes);

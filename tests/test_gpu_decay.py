@@ -1,5 +1,5 @@
 """The decay-gate quantiser at the edges of its walks: channel counts that are multiples of 128, of 64
-only, that divide 128, and others; 2 to 256 levels; few and odd numbers of rows; unaligned rates;
+only, that divide 128, others up to 256 and above; 2 to 256 levels; few and odd numbers of rows; unaligned rates;
 a rate that is not positive.  Codes bit for bit against the oracle."""
 import numpy as np
 import pytest
@@ -9,11 +9,12 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("row,H,dk", [(1, 1, 64), (1, 3, 64), (1, 2, 128), (1, 5, 128), (0, 1, 128), (0, 4, 128),
-                                      (0, 12, 128), (0, 16, 128), (0, 64, 64), (0, 192, 64), (0, 256, 64)])
+                                      (0, 2, 64), (0, 7, 128), (0, 12, 128), (0, 16, 128), (0, 61, 64), (0, 64, 64),
+                                      (0, 192, 64), (0, 250, 64), (0, 256, 64), (0, 257, 64)])
 @pytest.mark.parametrize("g", [1, 2, 3, 4, 5, 8])
 @pytest.mark.parametrize("B,T,pad", [(1, 1, 0), (2, 37, 0), (1, 641, 0), (3, 5, 1)])
 def test_quant_decay_walks(qs, orc, row, H, dk, g, B, T, pad):
-    cfg = qs.Config(B=B, H=H, dk=dk, dv=64, decay_kind=0 if row else 1, gate_bits=g)
+    cfg = qs.Config(B=B, H=H, dk=dk, dv=64, decay_kind=0 if row else 1, unit_kind=0 if row else 1, gate_bits=g)
     shape = (B, T, H, dk) if row else (B, T, H)
     chan, L = (H * dk if row else H), 1 << g
     rng = np.random.default_rng(H * 100 + g + T)
@@ -33,12 +34,13 @@ def test_quant_decay_walks(qs, orc, row, H, dk, g, B, T, pad):
     assert np.allclose(thr.cpu().numpy(), np.asarray(tref).reshape(-1), rtol=2.4e-7, atol=0)
 
 
-@pytest.mark.parametrize("row,H", [(1, 3), (0, 16), (0, 12)])
+@pytest.mark.parametrize("row,H", [(1, 3), (0, 16), (0, 12), (0, 7), (0, 257)])
+@pytest.mark.parametrize("at", [-1, -3])
 @pytest.mark.parametrize("bad", [0.0, -1.0, float("inf"), float("nan")])
-def test_quant_decay_rejects_bad_rates(qs, row, H, bad):
-    cfg = qs.Config(B=2, H=H, dk=128, dv=64, decay_kind=0 if row else 1, gate_bits=2)
+def test_quant_decay_rejects_bad_rates(qs, row, H, at, bad):
+    cfg = qs.Config(B=2, H=H, dk=128, dv=64, decay_kind=0 if row else 1, unit_kind=0 if row else 1, gate_bits=2)
     s = torch.rand((2, 9, H) + ((128,) if row else ()), device="cuda") + 0.1
-    s.view(-1)[-3] = bad
+    s.view(-1)[at] = bad
     chan = s[0, 0].numel()
     qs.qstate_quant_decay(cfg, s, torch.zeros(s.shape, dtype=torch.uint8, device="cuda"),
                           torch.zeros(chan * 4, device="cuda"), torch.zeros(chan * 3, device="cuda"))
