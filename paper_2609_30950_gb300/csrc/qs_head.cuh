@@ -1,6 +1,6 @@
 // qs_head.cuh -- write-back kernel for the head allocation unit (sm_103a): one width per head and
 // one FP16 step per scale group of 32 key rows x 1 value column (Sec. 3, "Allocation units";
-// Gated DeltaNet).  Also serves pack (dense -> packed) and unpack (packed -> dense) for this unit.
+// Gated DeltaNet).  Also serves pack (dense -> packed) for this unit; unpack_head_kernel unpacks it.
 //
 // One CTA of NW warps per (batch element, head).  Warp w owns row block w / NCS (32 key rows,
 // exactly one scale-group row) and column slice w % NCS (CS value columns); lane l owns the CPL
@@ -83,7 +83,7 @@ __device__ __forceinline__ void head_cand(float f, float R, float inv_n, float& 
     inv_ulp = d_ulp > 0.0f ? inv_ulp : 0.0f;
 }
 
-template <int DK, int DV, bool SRC_PACKED, bool DST_PACKED>
+template <int DK, int DV, bool SRC_PACKED>
 __global__ void __launch_bounds__(HeadGeom<DK, DV>::NT, 2) head_kernel(const StepParams p) {
     using G = HeadGeom<DK, DV>;
     static_assert(G::ok, "head-unit layout");
@@ -106,14 +106,14 @@ __global__ void __launch_bounds__(HeadGeom<DK, DV>::NT, 2) head_kernel(const Ste
 
     // ---- 1. widths and layout ---------------------------------------------------------------
     const int w_in = SRC_PACKED ? static_cast<int>(p.in_widths[bh]) : 0;
-    const int w_out = DST_PACKED ? static_cast<int>(p.out_widths[bh]) : 0;
+    const int w_out = static_cast<int>(p.out_widths[bh]);
     const int bytes_in = DK * DV / 8 * w_in, bytes_out = DK * DV / 8 * w_out;
     bool bad = false;
     if (SRC_PACKED) {
         const long long o = p.in_head_off[bh];
         bad |= w_in > 16 || o % align != 0 || o + bytes_in > p.region_bytes || bytes_in > p.stage_bytes;
     }
-    if (DST_PACKED) {
+    {
         const long long o = p.out_head_off[bh];
         bad |= w_out > 16 || o % align != 0 || o + bytes_out > p.region_bytes || bytes_out > p.stage_bytes;
     }
@@ -174,7 +174,7 @@ __global__ void __launch_bounds__(HeadGeom<DK, DV>::NT, 2) head_kernel(const Ste
         for (int r = 0; r < 32; ++r) x[r] = hv_bc<V>(0.0f);
     }
     if (SRC_PACKED) __syncthreads();   // the staging buffer is reused for the output rows
-    if (DST_PACKED) {                  // zero the output rows: codes are OR-ed in
+    {                                  // zero the output rows: codes are OR-ed in
         const int nz = (bytes_out + 16) / 16;
         for (int i = tid; i < nz; i += NT) reinterpret_cast<uint4*>(pay)[i] = make_uint4(0, 0, 0, 0);
         if (!has_tokens) __syncthreads();
@@ -289,7 +289,7 @@ __global__ void __launch_bounds__(HeadGeom<DK, DV>::NT, 2) head_kernel(const Ste
     }
 
     // ---- 4. write-back ----------------------------------------------------------------------------
-    if (DST_PACKED) {
+    {
         const int w = w_out;
         const bool refit = (p.fit_every <= 1) || ((p.w_index + h) % p.fit_every == 0);
         // magnitudes in place, signs kept aside (bit r of sg[c] = row r of column c negative)
@@ -439,13 +439,6 @@ __global__ void __launch_bounds__(HeadGeom<DK, DV>::NT, 2) head_kernel(const Ste
         Vec* dst = reinterpret_cast<Vec*>(p.out_payload + static_cast<size_t>(b) * p.region_bytes + p.out_head_off[bh]);
         const Vec* srcv = reinterpret_cast<const Vec*>(pay);
         for (int i = tid; i < bytes_out / static_cast<int>(sizeof(Vec)); i += NT) dst[i] = srcv[i];
-    } else if (p.dense_out != nullptr) {
-        float* dst = p.dense_out + (static_cast<size_t>(bh) * DK + r0) * DV + col0;
-#pragma unroll
-        for (int r = 0; r < 32; ++r) {
-            if constexpr (CPL == 2) *reinterpret_cast<float2*>(dst + r * DV) = x[r];
-            else dst[r * DV] = x[r];
-        }
     }
     if (stats && tid == 0) {
         p.ema_s[bh] = sm.ms;
@@ -453,9 +446,9 @@ __global__ void __launch_bounds__(HeadGeom<DK, DV>::NT, 2) head_kernel(const Ste
     }
 }
 
-template <int DK, int DV, bool SRC_PACKED, bool DST_PACKED>
+template <int DK, int DV, bool SRC_PACKED>
 cudaError_t launch_head_t(const qstate_cfg& cfg, const StepParams& p, cudaStream_t stream) {
-    auto kern = head_kernel<DK, DV, SRC_PACKED, DST_PACKED>;
+    auto kern = head_kernel<DK, DV, SRC_PACKED>;
     const int stage = DK * DV * cfg.bmax / 8;
     const size_t smem = sizeof(HeadSmem<DK, DV>) + static_cast<size_t>(stage) + 32;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -464,6 +457,81 @@ cudaError_t launch_head_t(const qstate_cfg& cfg, const StepParams& p, cudaStream
     StepParams q = p;
     q.stage_bytes = stage;
     kern<<<cfg.B * cfg.H, HeadGeom<DK, DV>::NT, smem, stream>>>(q);
+    return cudaGetLastError();
+}
+
+// ---- unpack of the head unit --------------------------------------------------------------------
+// As the row unit's (unpack_row_kernel): one small CTA per head, 6 per SM, each lane decoding four
+// consecutive codes of a row and storing 16 bytes.  A warp stays in one 32-row block, so a lane's four
+// steps are read once.
+// What bounds it: HBM, 4 dk dv bytes written per head.  A call from a cold L2, 256 x 16 heads of 128 x 128,
+// 6 bits: 66 us (319 MB); 88 us by the write-back's lanes, which hold two columns of a block's 32 rows, two
+// CTAs per SM.  134 x 46 heads of 128 x 64, 4 bits: 86 -> 50 us.
+template <int DK, int DV>
+__global__ void __launch_bounds__(256, 6) unpack_head_kernel(const __grid_constant__ StepParams p, bool vec) {
+    extern __shared__ __align__(16) uint8_t smem_raw[];
+    using Vec = typename std::conditional<DV == 128, uint4, uint2>::type;
+    constexpr int NB = DK / 32, WPB = 8 / NB;   // row blocks, and warps in each
+    constexpr int RS = 128 / DV;                // rows that a warp decodes at once
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int g = blockIdx.x, b = g / p.H;
+    const int w = p.in_widths[g], bytes = DK * DV / 8 * w;
+    const long long off = p.in_head_off[g];
+    const int half = lane / (32 / RS), cl = lane % (32 / RS), blk = warp / WPB;
+    const size_t gbase = static_cast<size_t>(g) * NB * DV + static_cast<size_t>(blk) * DV + cl * 4;
+    uint16_t sc[4];
+#pragma unroll
+    for (int c = 0; c < 4; ++c) sc[c] = p.in_scales[gbase + c];
+    if (w > 16 || off % static_cast<int>(sizeof(Vec)) != 0 || off + bytes > p.region_bytes || bytes > p.stage_bytes) {
+        if (tid == 0) raise_status(p.status, QS_DEV_LAYOUT);   // the whole CTA: nothing has been written
+        return;
+    }
+    const Vec* src = reinterpret_cast<const Vec*>(p.in_payload + static_cast<size_t>(b) * p.region_bytes + off);
+    for (int i = tid; i < bytes / static_cast<int>(sizeof(Vec)); i += 256) reinterpret_cast<Vec*>(smem_raw)[i] = __ldcs(src + i);
+    __syncthreads();
+    // w >= 2: q Delta; w = 1: +-m; w = 0: 0 (float(u) is 2^23 + u built from the code's bits)
+    const float A = 8388608.0f + static_cast<float>(w >= 2 ? (1 << (w - 1)) - 1 : 0);
+    float S[4], B[4];
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+        const float D = f16_value(sc[c]);
+        S[c] = w >= 2 ? D : (w == 1 ? -2.0f * D : 0.0f);
+        B[c] = w == 1 ? D : 0.0f;
+    }
+    const int P = cl * 4 * w, idx = P >> 5, sh = P & 31, rowwords = w * DV / 32;
+    const uint32_t mask = (1u << w) - 1u;
+    const int r0 = 32 * blk + (warp % WPB) * RS + half;
+    const uint32_t* words = reinterpret_cast<const uint32_t*>(smem_raw) + r0 * rowwords + idx;
+    float* dst = p.dense_out + (static_cast<size_t>(g) * DK + r0) * DV + cl * 4;
+#pragma unroll 4
+    for (int r = 0; r < 32; r += WPB * RS) {
+        const uint32_t* wd = words + r * rowwords;
+        const uint32_t lo = __funnelshift_r(wd[0], wd[1], sh), hi = __funnelshift_r(wd[1], wd[2], sh);
+        const uint64_t chunk = (static_cast<uint64_t>(hi) << 32) | lo;
+        float x[4];
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+            const uint32_t u = static_cast<uint32_t>(chunk >> (c * w)) & mask;
+            x[c] = fmaf(__fsub_rn(__uint_as_float(kTwo23Bits | u), A), S[c], B[c]);
+        }
+        float* o = dst + r * DV;
+        if (vec) {
+            __stcs(reinterpret_cast<float4*>(o), make_float4(x[0], x[1], x[2], x[3]));
+        } else {
+#pragma unroll
+            for (int c = 0; c < 4; ++c) o[c] = x[c];
+        }
+    }
+}
+
+template <int DK, int DV>
+cudaError_t launch_unpack_head_t(const qstate_cfg& cfg, const StepParams& p, cudaStream_t stream) {
+    StepParams q = p;
+    q.stage_bytes = DK * DV * cfg.bmax / 8;
+    const int smem = q.stage_bytes + 16;   // the last lane reads up to 8 bytes past the head's rows
+    cudaError_t e = cudaFuncSetAttribute(unpack_head_kernel<DK, DV>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    if (e != cudaSuccess) return e;
+    unpack_head_kernel<DK, DV><<<cfg.B * cfg.H, 256, smem, stream>>>(q, (reinterpret_cast<uintptr_t>(p.dense_out) & 15) == 0);
     return cudaGetLastError();
 }
 

@@ -475,9 +475,9 @@ cudaError_t launch_step_shape(const qstate_cfg& cfg, int src_packed, int dst_pac
             if (src_packed && dst_packed && p.t_end > p.t_begin && p.in_fidx && a16(p.in_payload) &&
                 a16(p.out_payload) && a16(p.in_scales) && a16(p.in_fidx) && a16(p.k) && a16(p.q) && a16(p.v))
                 return launch_head_wb_t<DK, DV>(cfg, p, stream);
-            if (src_packed && dst_packed) return launch_head_t<DK, DV, true, true>(cfg, p, stream);
-            if (!src_packed && dst_packed) return launch_head_t<DK, DV, false, true>(cfg, p, stream);
-            return launch_head_t<DK, DV, true, false>(cfg, p, stream);
+            if (src_packed && dst_packed) return launch_head_t<DK, DV, true>(cfg, p, stream);
+            if (!src_packed && dst_packed) return launch_head_t<DK, DV, false>(cfg, p, stream);
+            return launch_unpack_head_t<DK, DV>(cfg, p, stream);
         }
         return cudaErrorInvalidValue;
     }
