@@ -70,7 +70,7 @@ def algorithmic_bytes(w, fit_every=1):
 
 # Committed ncu summaries that carry a DRAM traffic figure, per (workload, interval form):
 # the summary and the kernel sources its figure was taken on.
-_CORE = ("qs_wb_row.cuh", "qs_common.cuh", "qs_internal.h")
+_CORE = ("qs_wb_row.cuh", "qs_rowquant.cuh", "qs_common.cuh", "qs_internal.h")
 TRAFFIC_PROFILES = {
     ("kda_decode", "token"): ("writeback_kda_decode.md", _CORE),
     ("kda_prefill", "chunk"): ("writeback_kda_prefill_chunk.md", _CORE + ("qs_chunk.cuh", "qs_tc.cuh")),

@@ -4,7 +4,7 @@
 // interval of every head, packed state in, packed state out.
 //
 // Each CTA (NW = 8 warps, two CTAs per SM so that one's barriers and latencies overlap the
-// other's work) walks a contiguous block of heads.  While it works on head g, cp.async copies
+// other's work; the chunked form 16 warps and one CTA per SM) walks a contiguous block of heads.  While it works on head g, cp.async copies
 // head g + 1's metadata into the other half of a double buffer (widths in/out, FP16 scales,
 // fitted-factor indices, EMA statistics, the first token's k, q, v, rates and their level
 // table; issued by the one warp without a prep role) and, once head g's tokens are done, head
