@@ -22,7 +22,7 @@ _HERE = os.path.dirname(os.path.abspath(__file__))
 _SRC = os.path.join(_HERE, "qstate_oracle.c")
 _LIB = os.path.join(_HERE, "_build", "liborc.so")
 # timing build: the same source with a write-back's heads shared out over OpenMP threads
-# (identical arithmetic per head); the checker is always the plain single-thread build
+# (identical arithmetic per head); the oracle is always the plain single-thread build
 _LIB_OMP = os.path.join(_HERE, "_build", "liborc_omp.so")
 _FLAGS = ["-std=c11", "-O2", "-ffp-contract=off", "-fno-fast-math", "-fPIC", "-shared"]
 
@@ -112,7 +112,7 @@ _lib_par = None
 
 
 def lib(parallel: bool = False):
-    """The plain build (the checker), or with ``parallel`` the OpenMP timing build."""
+    """The plain build (the oracle), or with ``parallel`` the OpenMP timing build."""
     global _lib, _lib_par
     if parallel:
         if _lib_par is None:
