@@ -206,9 +206,12 @@ bool aligned16(const void* ptr) { return (reinterpret_cast<uintptr_t>(ptr) & 15u
 // every per-head array 16-byte aligned; otherwise the one-head-per-CTA kernel runs.
 bool wb_row_eligible(const qstate_cfg& c, const StepParams& p) {
     if (c.unit_kind != QSTATE_UNIT_ROW) return false;
+    // (the level table is copied for row codes of up to 4 levels, a and w under general erasure)
+    const bool lut = p.decay_row && p.s_code && p.L <= 4;
     const void* ptrs[] = {p.in_payload, p.in_scales, p.in_widths, p.in_fidx, p.out_payload,
                           p.out_widths, p.q, p.k, p.v, p.ema_s, p.ema_r,
-                          p.s_code ? static_cast<const void*>(p.s_code) : static_cast<const void*>(p.s)};
+                          p.s_code ? static_cast<const void*>(p.s_code) : static_cast<const void*>(p.s),
+                          lut ? p.s_lut : nullptr, p.general ? p.a_in : nullptr, p.general ? p.w_in : nullptr};
     for (const void* q : ptrs)
         if (q && !aligned16(q)) return false;
     if (!p.in_fidx) return false;

@@ -1,0 +1,55 @@
+"""Write-backs whose arrays do not begin on a 16-byte boundary (views into larger tensors), in lockstep
+with the oracle: such calls take the kernels without 16-byte copies and compute the same."""
+import pytest
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+import synth  # noqa: E402
+from test_gpu_parity import _lockstep  # noqa: E402
+
+WORKLOADS = {**synth.WORKLOADS, **synth.EXTENSION_WORKLOADS}
+
+
+class Shifted:
+    """The binding with the named arrays one element past a 16-byte boundary."""
+
+    def __init__(self, qs, *names):
+        self.qs, self.names = qs, set(names)
+
+    def __getattr__(self, name):
+        return getattr(self.qs, name)
+
+    def shift(self, obj):
+        for n in self.names & set(vars(obj)):
+            t = getattr(obj, n)
+            if t is not None:
+                buf = torch.zeros(t.numel() + 1, dtype=t.dtype, device=t.device)
+                buf[1:] = t.reshape(-1)
+                setattr(obj, n, buf[1:].view(t.shape))
+                assert getattr(obj, n).data_ptr() % 16 == t.element_size()
+        return obj
+
+    def Inputs(self, *args):
+        return self.shift(self.qs.Inputs(*args))
+
+    def new_state(self, cfg):
+        return self.shift(self.qs.new_state(cfg))
+
+    def new_stats(self, cfg):
+        return self.shift(self.qs.new_stats(cfg))
+
+
+@pytest.mark.parametrize("dk,dv", [(128, 128), (128, 64), (64, 64)])
+@pytest.mark.parametrize("name,array,C", [("kda_general", "a", 1), ("kda_general", "w", 3), ("kda_decode", "s_lut", 1),
+                                          ("kda_decode", "s_lut", 5)])
+def test_one_token_input(qs, orc, dk, dv, name, array, C):
+    """a, w and the level table, which the 16-byte kernel copies too."""
+    w = synth.scaled(WORKLOADS[name], B=2, H=3, T=10, C=C, dk=dk, dv=dv)
+    _lockstep(Shifted(qs, array), orc, w, log_decay=array == "s_lut")
+
+
+def test_level_table_chunked(qs, orc):
+    """The chunked form copies the level table too: without its alignment the token form runs."""
+    w = synth.scaled(WORKLOADS["kda_prefill"], B=1, H=2, T=70, C=48, gate_bits=2)
+    _lockstep(Shifted(qs, "s_lut"), orc, w, log_decay=True, interval_form=1)
