@@ -120,7 +120,8 @@ typedef struct qstate_cfg {
  *           head_off[b*H + h]; its rows follow in order, row i taking width_i*dv/8 bytes; row
  *           element j's code occupies row bits [j*w, j*w + w), bit m of a row being bit m%8
  *           of byte m/8.  Codes: w >= 2 -> offset binary q + n, n = 2^(w-1) - 1; w = 1 ->
- *           sign bit (1 = negative); w = 0 -> nothing stored.
+ *           sign bit (1 = negative); w = 0 -> nothing stored.  The base is 16-byte aligned at
+ *           dv = 128 and 8-byte aligned at dv = 64 (else EINVAL).
  *  scales   FP16 bit patterns, one per scale group: (B, H, dk) for the row unit, (B, H, dk/32,
  *           dv) for the head unit.  w >= 2: step Delta; w = 1: mean |x|.
  *  widths   uint8, (B, H, dk) for the row unit, (B, H) for the head unit.

@@ -193,6 +193,15 @@ bool buf_ok(const qstate_buf* b) {
     return b && b->payload && b->scales && b->widths && b->head_off && b->fidx;
 }
 
+// Every kernel moves a row's or head's payload in 16-byte (dv = 128) or 8-byte words; regions and
+// offsets keep that alignment, so the base has to have it.
+int check_payload(const qstate_cfg* c, const qstate_buf* b) {
+    const uintptr_t need = c->dv == 128 ? 16 : 8;
+    if (reinterpret_cast<uintptr_t>(b->payload) % need != 0)
+        return fail(QSTATE_EINVAL, "payload must be %d-byte aligned at dv = %d", static_cast<int>(need), c->dv);
+    return QSTATE_OK;
+}
+
 cudaError_t launch_step_any(const qstate_cfg& c, int src_packed, int dst_packed, const StepParams& p,
                             cudaStream_t st) {
     if (c.dk == 128 && c.dv == 128) return launch_step_128x128(c, src_packed, dst_packed, p, st);
@@ -476,6 +485,7 @@ int step(const qstate_cfg* cfg, qstate_buf* in, qstate_buf* out, const qstate_in
     int rc = validate(cfg);
     if (rc) return rc;
     if (!buf_ok(in) || !buf_ok(out)) return fail(QSTATE_EINVAL, "null buffer pointer");
+    if ((rc = check_payload(cfg, in)) || (rc = check_payload(cfg, out))) return rc;
     if (!stats || !stats->ema_s || !stats->ema_r || (cfg->unit_kind == QSTATE_UNIT_ROW && !stats->range))
         return fail(QSTATE_EINVAL, "null statistics pointer");
     if ((rc = check_inputs(cfg, x, t_begin, t_end, o))) return rc;
@@ -556,6 +566,7 @@ int qstate_init(const qstate_cfg* cfg, qstate_buf* a, qstate_buf* b, void* strea
     int rc = validate(cfg);
     if (rc) return rc;
     if (!buf_ok(a) || !buf_ok(b)) return fail(QSTATE_EINVAL, "null buffer pointer");
+    if ((rc = check_payload(cfg, a))) return rc;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     int* status = nullptr;
     if ((rc = acquire_status(&status))) return rc;
@@ -597,6 +608,7 @@ int qstate_pack(const qstate_cfg* cfg, const float* S, qstate_buf* out, float* r
     int rc = validate(cfg);
     if (rc) return rc;
     if (!S || !buf_ok(out)) return fail(QSTATE_EINVAL, "null pointer");
+    if ((rc = check_payload(cfg, out))) return rc;
     int* status = nullptr;
     if ((rc = acquire_status(&status))) return rc;
     cudaError_t e;
@@ -617,6 +629,7 @@ int qstate_unpack(const qstate_cfg* cfg, const qstate_buf* in, float* S_out, voi
     int rc = validate(cfg);
     if (rc) return rc;
     if (!S_out || !buf_ok(in)) return fail(QSTATE_EINVAL, "null pointer");
+    if ((rc = check_payload(cfg, in))) return rc;
     int* status = nullptr;
     if ((rc = acquire_status(&status))) return rc;
     cudaError_t e;

@@ -74,6 +74,27 @@ def test_calls_reject_null_pointers_without_launching(lib):
     assert b"null" in lib.qstate_last_error()
 
 
+@pytest.mark.parametrize("dk,dv,off", [(128, 128, 8), (128, 128, 4), (128, 64, 4), (64, 64, 1)])
+@pytest.mark.parametrize("head", [0, 1])
+def test_payload_off_its_boundary_is_refused_without_launching(lib, dk, dv, off, head):
+    """Placeholder device addresses, which the calls refuse before anything could read them."""
+    import paper_2609_30950_gb300 as q
+    cfg = q.Config(B=1, H=2, dk=dk, dv=dv, decay_kind=head, unit_kind=head).c()
+    A = 1 << 20
+    good, bad = q._Buf(A, A, A, A, A), q._Buf(A + off, A, A, A, A)
+    x, st = q._Inputs(A, A, A, A, None, None, A, 1, None, None), q._Stats(A, A, A)
+    r = ct.byref
+    flag = ct.c_int32(0)
+    calls = [lambda: lib.qstate_init(r(cfg), r(bad), r(good), None), lambda: lib.qstate_pack(r(cfg), A, r(bad), None, None),
+             lambda: lib.qstate_unpack(r(cfg), r(bad), A, None),
+             lambda: lib.qstate_step(r(cfg), r(bad), r(good), r(x), 0, 1, 0, A, r(st), None),
+             lambda: lib.qstate_step(r(cfg), r(good), r(bad), r(x), 0, 1, 0, A, r(st), None),
+             lambda: lib.qstate_scan(r(cfg), r(good), r(bad), r(x), 0, 1, 0, A, r(st), r(flag), None)]
+    for call in calls:
+        assert call() == q.QSTATE_EINVAL
+        assert b"aligned" in lib.qstate_last_error()
+
+
 def test_chunked_form_configuration_limits(lib):
     """The chunked form (interval_form = 1) is for the row unit at dk = dv = 128 with the
     delta rule or no erasure; anything else is rejected before a launch."""
