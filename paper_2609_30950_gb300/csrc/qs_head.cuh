@@ -164,10 +164,15 @@ __global__ void __launch_bounds__(HeadGeom<DK, DV>::NT, 2) head_kernel(const Ste
         }
     } else if (p.dense_in != nullptr) {
         const float* src = p.dense_in + (static_cast<size_t>(bh) * DK + r0) * DV + col0;
+        if (CPL == 2 && (reinterpret_cast<uintptr_t>(src) & 7) == 0) {
 #pragma unroll
-        for (int r = 0; r < 32; ++r) {
-            if constexpr (CPL == 2) x[r] = *reinterpret_cast<const float2*>(src + r * DV);
-            else x[r] = src[r * DV];
+            for (int r = 0; r < 32; ++r)
+                if constexpr (CPL == 2) x[r] = *reinterpret_cast<const float2*>(src + r * DV);
+        } else {
+#pragma unroll
+            for (int r = 0; r < 32; ++r)
+#pragma unroll
+                for (int c = 0; c < CPL; ++c) hv_set(x[r], c, src[r * DV + c]);
         }
     } else {
 #pragma unroll

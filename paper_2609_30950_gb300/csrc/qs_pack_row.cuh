@@ -29,9 +29,9 @@ struct alignas(16) PackSmem {
     int flag, next;
 };
 
-// vec: the dense state is 16-byte aligned (else 8).
+// align: the dense state's alignment, 16, 8 or 4 bytes.
 template <int DK, int DV>
-__global__ void __launch_bounds__(128, 4) pack_row_kernel(const __grid_constant__ StepParams p, bool vec) {
+__global__ void __launch_bounds__(128, 4) pack_row_kernel(const __grid_constant__ StepParams p, int align) {
     using RQ = RowQuant<DV>;
     constexpr int TPR = RQ::TPR, RPB = RQ::RPB, NB = DK / RPB, NW = PackSmem<DK, DV>::NW;
     __shared__ PackSmem<DK, DV> sm;
@@ -96,13 +96,16 @@ __global__ void __launch_bounds__(128, 4) pack_row_kernel(const __grid_constant_
             const float* src = p.dense_in + (rb + i) * DV + 32 * q;
 #pragma unroll
             for (int c = 0; c < 8; ++c) {
-                if (vec) {
+                if (align == 16) {
                     const float4 v = __ldcs(reinterpret_cast<const float4*>(src + 4 * c));
                     xv[2 * c] = make_float2(v.x, v.y);
                     xv[2 * c + 1] = make_float2(v.z, v.w);
-                } else {
+                } else if (align == 8) {
                     xv[2 * c] = *reinterpret_cast<const float2*>(src + 4 * c);
                     xv[2 * c + 1] = *reinterpret_cast<const float2*>(src + 4 * c + 2);
+                } else {
+                    xv[2 * c] = make_float2(src[4 * c], src[4 * c + 1]);
+                    xv[2 * c + 1] = make_float2(src[4 * c + 2], src[4 * c + 3]);
                 }
             }
         } else {
@@ -157,7 +160,8 @@ template <int DK, int DV>
 cudaError_t launch_pack_row_t(const qstate_cfg& cfg, const StepParams& p, cudaStream_t stream) {
     StepParams q = p;
     q.stage_bytes = DK * DV * cfg.bmax / 8;
-    pack_row_kernel<DK, DV><<<cfg.B * cfg.H, 128, 0, stream>>>(q, (reinterpret_cast<uintptr_t>(p.dense_in) & 15) == 0);
+    const uintptr_t at = reinterpret_cast<uintptr_t>(p.dense_in);
+    pack_row_kernel<DK, DV><<<cfg.B * cfg.H, 128, 0, stream>>>(q, at % 16 == 0 ? 16 : at % 8 == 0 ? 8 : 4);
     return cudaGetLastError();
 }
 
@@ -167,7 +171,8 @@ cudaError_t launch_pack_row_t(const qstate_cfg& cfg, const StepParams& p, cudaSt
 // stores going.  The payload window is taken from the neighbouring head offsets so that its copy
 // does not wait for the sum of the widths; if the widths ask for more, the rest is copied after.
 // Lanes decode four consecutive codes and store 16 bytes; at dv = 64 the half-warps take
-// alternate rows.
+// alternate rows.  A dense state that is not 16-byte aligned: every 32nd (16th) column to a lane, so that
+// its 4-byte stores have no gaps.
 // What bounds it: HBM, 64 KB written per head.  64 x 32 heads of 128 x 128, 4 bits: 26.6 us (151 MB,
 // 5.7 TB/s); 45 us with two CTAs of 256 threads per SM, whose loads, prefix sum and stores followed one
 // another.
@@ -238,6 +243,22 @@ __global__ void __launch_bounds__(256, 6) unpack_row_kernel(const __grid_constan
     }
     constexpr int RS = 128 / DV;   // rows that a warp decodes at once
     const int half = lane / (32 / RS), cl = lane % (32 / RS);
+    if (!vec) {
+#pragma unroll 2
+        for (int r = warp * RS + half; r < DK; r += 8 * RS) {
+            const float4 dq = sm.deq[r];
+            const int w = __float_as_int(dq.w);
+            const uint32_t* words = reinterpret_cast<const uint32_t*>(pay + sm.off[r]);
+            float* o = p.dense_out + (rb + r) * DV;
+#pragma unroll
+            for (int col = cl; col < DV; col += 32 / RS) {
+                const int P = col * w, idx = P >> 5;
+                const uint32_t u = __funnelshift_r(words[idx], words[idx + 1], P & 31) & ((1u << w) - 1u);
+                o[col] = fmaf(__fsub_rn(__uint_as_float(kTwo23Bits | u), dq.x), dq.y, dq.z);
+            }
+        }
+        return;
+    }
     float* dst = p.dense_out + rb * DV + cl * 4;
 #pragma unroll 4
     for (int r = warp * RS + half; r < DK; r += 8 * RS) {
@@ -255,13 +276,7 @@ __global__ void __launch_bounds__(256, 6) unpack_row_kernel(const __grid_constan
             const uint32_t u = static_cast<uint32_t>(chunk >> (c * w)) & mask;
             x[c] = fmaf(__fsub_rn(__uint_as_float(kTwo23Bits | u), dq.x), dq.y, dq.z);
         }
-        float* o = dst + r * DV;
-        if (vec) {
-            __stcs(reinterpret_cast<float4*>(o), make_float4(x[0], x[1], x[2], x[3]));
-        } else {
-            *reinterpret_cast<float2*>(o) = make_float2(x[0], x[1]);
-            *reinterpret_cast<float2*>(o + 2) = make_float2(x[2], x[3]);
-        }
+        __stcs(reinterpret_cast<float4*>(dst + r * DV), make_float4(x[0], x[1], x[2], x[3]));
     }
 }
 

@@ -53,3 +53,36 @@ def test_level_table_chunked(qs, orc):
     """The chunked form copies the level table too: without its alignment the token form runs."""
     w = synth.scaled(WORKLOADS["kda_prefill"], B=1, H=2, T=70, C=48, gate_bits=2)
     _lockstep(Shifted(qs, "s_lut"), orc, w, log_decay=True, interval_form=1)
+
+
+@pytest.mark.parametrize("dk,dv", [(128, 128), (128, 64), (64, 64)])
+@pytest.mark.parametrize("head", [0, 1])
+@pytest.mark.parametrize("pad", [1, 2, 3])
+def test_dense_state(qs, dk, dv, head, pad):
+    """Pack from and unpack to a dense state at any 4-byte alignment: as with an aligned one."""
+    B, H = 2, 17
+    cfg = qs.Config(B=B, H=H, dk=dk, dv=dv, decay_kind=head, unit_kind=head, bbar_num=8, bbar_den=1, bmin=0, bmax=16)
+    gen = torch.Generator(device="cuda").manual_seed(dk + dv + pad)
+    S = torch.randn((B, H, dk, dv), device="cuda", generator=gen)
+    # widths 0 to 16, over the rows of a head or over the heads
+    w = (torch.arange(17, dtype=torch.uint8).repeat(B) if head else
+         torch.stack([torch.arange(dk) % 17 for _ in range(B * H)]).clamp(max=16).to(torch.uint8).reshape(-1))
+    per_head = (w.view(B, H, -1).int().sum(2) * (dk * dv if head else dv) // 8).cpu()
+    assert int(per_head.sum(1).max()) <= qs.region_bytes(cfg)
+    off = torch.cumsum(per_head, 1).int() - per_head.int()
+    got = []
+    for p in (0, pad):
+        st = qs.new_state(cfg)
+        st.widths.copy_(w)
+        st.head_off.copy_(off.reshape(-1))
+        buf = torch.full((S.numel() + p + 4,), 7.0, device="cuda")
+        view = buf[p:p + S.numel()].view(S.shape)
+        view.copy_(S)
+        qs.qstate_pack(cfg, view, st)
+        view.fill_(0)
+        qs.qstate_unpack(cfg, st, view)
+        qs.qstate_check()
+        assert bool((buf[:p] == 7).all()) and bool((buf[p + S.numel():] == 7).all())
+        got.append((st.payload, st.scales, st.fidx, view.clone()))
+    for a, b in zip(*got):
+        assert torch.equal(a, b)
