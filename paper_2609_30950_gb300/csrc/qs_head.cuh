@@ -471,7 +471,9 @@ cudaError_t launch_head_t(const qstate_cfg& cfg, const StepParams& p, cudaStream
 // steps are read once.
 // What bounds it: HBM, 4 dk dv bytes written per head.  A call from a cold L2, 256 x 16 heads of 128 x 128,
 // 6 bits: 66 us (319 MB); 88 us by the write-back's lanes, which hold two columns of a block's 32 rows, two
-// CTAs per SM.  134 x 46 heads of 128 x 64, 4 bits: 86 -> 50 us.
+// CTAs per SM.  134 x 46 heads of 128 x 64, 4 bits: 86 -> 50 us.  A dense state that is not 16-byte aligned:
+// every 32nd (16th) column to a lane, whose 4-byte stores then have no gaps (512 heads
+// of 128 x 64, 4 bits: 6.0 us; 9.2 with four consecutive columns, 7.2 by the write-back's lanes).
 template <int DK, int DV>
 __global__ void __launch_bounds__(256, 6) unpack_head_kernel(const __grid_constant__ StepParams p, bool vec) {
     extern __shared__ __align__(16) uint8_t smem_raw[];
@@ -482,11 +484,13 @@ __global__ void __launch_bounds__(256, 6) unpack_head_kernel(const __grid_consta
     const int g = blockIdx.x, b = g / p.H;
     const int w = p.in_widths[g], bytes = DK * DV / 8 * w;
     const long long off = p.in_head_off[g];
-    const int half = lane / (32 / RS), cl = lane % (32 / RS), blk = warp / WPB;
-    const size_t gbase = static_cast<size_t>(g) * NB * DV + static_cast<size_t>(blk) * DV + cl * 4;
+    constexpr int CW = 32 / RS;                 // lanes over a row
+    const int half = lane / CW, cl = lane % CW, blk = warp / WPB;
+    // the lane's columns: 4 cl .. 4 cl + 3, or cl + c CW
+    const size_t gbase = static_cast<size_t>(g) * NB * DV + static_cast<size_t>(blk) * DV;
     uint16_t sc[4];
 #pragma unroll
-    for (int c = 0; c < 4; ++c) sc[c] = p.in_scales[gbase + c];
+    for (int c = 0; c < 4; ++c) sc[c] = p.in_scales[gbase + (vec ? cl * 4 + c : cl + c * CW)];
     if (w > 16 || off % static_cast<int>(sizeof(Vec)) != 0 || off + bytes > p.region_bytes || bytes > p.stage_bytes) {
         if (tid == 0) raise_status(p.status, QS_DEV_LAYOUT);   // the whole CTA: nothing has been written
         return;
@@ -503,14 +507,28 @@ __global__ void __launch_bounds__(256, 6) unpack_head_kernel(const __grid_consta
         S[c] = w >= 2 ? D : (w == 1 ? -2.0f * D : 0.0f);
         B[c] = w == 1 ? D : 0.0f;
     }
-    const int P = cl * 4 * w, idx = P >> 5, sh = P & 31, rowwords = w * DV / 32;
+    const int rowwords = w * DV / 32;
     const uint32_t mask = (1u << w) - 1u;
     const int r0 = 32 * blk + (warp % WPB) * RS + half;
-    const uint32_t* words = reinterpret_cast<const uint32_t*>(smem_raw) + r0 * rowwords + idx;
-    float* dst = p.dense_out + (static_cast<size_t>(g) * DK + r0) * DV + cl * 4;
+    const uint32_t* words = reinterpret_cast<const uint32_t*>(smem_raw) + r0 * rowwords;
+    float* dst = p.dense_out + (static_cast<size_t>(g) * DK + r0) * DV;
+    if (!vec) {
+#pragma unroll 2
+        for (int r = 0; r < 32; r += WPB * RS) {
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+                const int col = cl + c * CW, P = col * w;
+                const uint32_t* wd = words + r * rowwords + (P >> 5);
+                const uint32_t u = __funnelshift_r(wd[0], wd[1], P & 31) & mask;
+                dst[r * DV + col] = fmaf(__fsub_rn(__uint_as_float(kTwo23Bits | u), A), S[c], B[c]);
+            }
+        }
+        return;
+    }
+    const int P = cl * 4 * w, idx = P >> 5, sh = P & 31;
 #pragma unroll 4
     for (int r = 0; r < 32; r += WPB * RS) {
-        const uint32_t* wd = words + r * rowwords;
+        const uint32_t* wd = words + r * rowwords + idx;
         const uint32_t lo = __funnelshift_r(wd[0], wd[1], sh), hi = __funnelshift_r(wd[1], wd[2], sh);
         const uint64_t chunk = (static_cast<uint64_t>(hi) << 32) | lo;
         float x[4];
@@ -519,13 +537,7 @@ __global__ void __launch_bounds__(256, 6) unpack_head_kernel(const __grid_consta
             const uint32_t u = static_cast<uint32_t>(chunk >> (c * w)) & mask;
             x[c] = fmaf(__fsub_rn(__uint_as_float(kTwo23Bits | u), A), S[c], B[c]);
         }
-        float* o = dst + r * DV;
-        if (vec) {
-            __stcs(reinterpret_cast<float4*>(o), make_float4(x[0], x[1], x[2], x[3]));
-        } else {
-#pragma unroll
-            for (int c = 0; c < 4; ++c) o[c] = x[c];
-        }
+        __stcs(reinterpret_cast<float4*>(dst + r * DV + cl * 4), make_float4(x[0], x[1], x[2], x[3]));
     }
 }
 
