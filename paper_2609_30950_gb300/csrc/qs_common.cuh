@@ -23,10 +23,14 @@ constexpr uint32_t kTwo23Bits = 0x4B000000u;
 // Start of a kernel launched by launch_chained: waits until the launches before it in the stream are
 // complete and their writes visible (nothing global is touched before, and nothing after through
 // the read-only path, whose data must not change while a kernel runs), then lets the one after
-// it take its place on idle SMs.
+// it take its place on idle SMs.  A kernel that takes tensor memory takes it between the two: taken
+// before the wait, a kernel that is waited for might need those columns; taken after the release, the
+// one released might take them first and wait for this one.
+__device__ __forceinline__ void chain_enter() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void chain_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void chain_wait() {
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    chain_enter();
+    chain_release();
 }
 
 // Record a QS_DEV_* condition in the status word (one per device, see qs_api.cu).

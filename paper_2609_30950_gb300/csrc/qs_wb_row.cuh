@@ -271,8 +271,9 @@ __global__ void __launch_bounds__(NW * 32, CHUNK ? 1 : 2) wb_row_kernel(const Wb
     const int g_end = static_cast<int>(static_cast<long long>(blockIdx.x + 1) * wp.nheads / gridDim.x);
     uint8_t* cb = pay + ((p.stage_bytes + 32 + 15) & ~15);   // chunked form's region
     uint32_t tmem = 0, mphase = 0;
+    chain_enter();
     if constexpr (CHUNK) tmem = chunk_setup(cb);
-    chain_wait();
+    chain_release();
     {
         const int h0 = g_begin % p.H;
         const int io = static_cast<int>(p.in_head_off[g_begin]);

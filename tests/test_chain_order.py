@@ -1,0 +1,20 @@
+"""Orders within the kernels that no run can show to be missing, read from the sources."""
+import os
+import re
+
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2609_30950_gb300", "csrc")
+
+
+def source(name):
+    text = open(os.path.join(CSRC, name)).read()
+    return re.sub(r"//[^\n]*", "", text)
+
+
+def test_tensor_memory_is_taken_between_wait_and_release():
+    """A chained launch that held tensor memory while it waits could starve the kernel it waits for, and
+    one that let its dependents start before it holds its own could be starved by them."""
+    src = source("qs_wb_row.cuh")
+    body = src[src.index("wb_row_kernel(const WbParams wp)"):]
+    at = [body.index(s) for s in ("chain_enter();", "chunk_setup(cb)", "chain_release();", "wb_issue_meta<DK, DV>(sm.st[0]")]
+    assert at == sorted(at)
+    assert body.count("chain_") == 2 and "chain_wait" not in src
