@@ -541,9 +541,9 @@ __device__ __forceinline__ void chunk_interval(const StepParams& p, Stage& S, fl
         }
         tc::fence_before_sync();
         __syncthreads();                                                            // C3
+        tc::fence_after_sync();   // every thread reads u, which warps 4-7 wrote
         // update = u^T (k o Dc_{L-1} / Dc) on the tensor cores (3xTF32, K = 16 tokens)
         if (tid == 0) {
-            tc::fence_after_sync();
             constexpr uint32_t idU = tc::idesc_tf32(128, D);
             constexpr uint64_t kStepU = (2 * G::kLboU) >> 4;
             uint64_t bh = tc::smem_desc(tc::smem_addr(bu_hi), G::kLboU, G::kSboU);
