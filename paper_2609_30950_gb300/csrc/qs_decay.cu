@@ -35,7 +35,7 @@ __global__ void decay_init_kernel(float* lut, int nchan, int L) {
 // How a launch walks the rates 16 bytes at a time: LC lanes cover P = 4 LC consecutive values, a
 // chunk of one row's channels (P divides nchan) or several whole rows (nchan divides P), so a lane's
 // channels are fixed; 256 / LC such strips per block step through the strips of its chunk.  Other
-// channel counts up to kAnyChannels (ANY, one chunk) take a number of blocks for which the step is a
+// channel counts (ANY, one chunk) take a number of blocks for which the step is a
 // multiple of nchan: a lane's channels are fixed too, but differ between the strips of a block.
 struct Walk {
     long long total, pitch;   // values in whole groups of 4; between a chunk's consecutive strips
@@ -43,7 +43,7 @@ struct Walk {
     int chunks, nchan;
     int tail;                 // values after the whole groups (0 to 3), by the first block's first threads
 };
-constexpr int kAnyChannels = 256;
+constexpr int kAnyChannels = 1024;   // heads, at most
 constexpr int kDecayThreads = 256, kInFlight = 4;
 // Blocks per SM, all resident, so that the sweeps keep their order: by the registers that the
 // thresholds take.
@@ -117,16 +117,25 @@ __global__ void __launch_bounds__(kDecayThreads, kMinmaxBlocks) decay_minmax_row
     const int nc = ANY ? wk.nchan : min(wk.nchan, 4 * LC);
     if constexpr (ANY) {
         // the block's values follow one another from a multiple of 1024 on: every nc-th is a channel's
-        const int per = kDecayThreads / nc, t = threadIdx.x;
-        if (t < per * nc) {
-            uint32_t lo = ~0u, hi = 0u;
-            for (int i = t; i < 4 * kDecayThreads; i += per * nc) {
-                lo = min(lo, vmn[i]);
-                hi = max(hi, vmx[i]);
+        const long long first = static_cast<long long>(blockIdx.x) * 4 * kDecayThreads;
+        if (nc <= kDecayThreads) {
+            const int per = kDecayThreads / nc * nc, t = threadIdx.x;
+            if (t < per) {
+                uint32_t lo = ~0u, hi = 0u;
+                for (int i = t; i < 4 * kDecayThreads; i += per) {
+                    lo = min(lo, vmn[i]);
+                    hi = max(hi, vmx[i]);
+                }
+                const int ch = static_cast<int>((first + t) % nc);
+                atomicMin(&cmn[ch], lo);
+                atomicMax(&cmx[ch], hi);
             }
-            const int ch = static_cast<int>((static_cast<long long>(blockIdx.x) * 4 * kDecayThreads + t) % nc);
-            atomicMin(&cmn[ch], lo);
-            atomicMax(&cmx[ch], hi);
+        } else {
+            for (int i = threadIdx.x; i < 4 * kDecayThreads; i += kDecayThreads) {
+                const int ch = static_cast<int>((first + i) % nc);
+                atomicMin(&cmn[ch], vmn[i]);
+                atomicMax(&cmx[ch], vmx[i]);
+            }
         }
     } else {
         for (int i = threadIdx.x; i < 4 * LC; i += kDecayThreads) {
@@ -148,14 +157,15 @@ __global__ void __launch_bounds__(kDecayThreads, kMinmaxBlocks) decay_minmax_row
     }
     __syncthreads();
     for (int i = threadIdx.x; i < nc; i += kDecayThreads) {
+        if (cmx[i] == 0u) continue;   // no good rate of this channel here
         float* l = lut + (static_cast<size_t>(chunk) * 4 * LC + i) * L;
         atomicMin(reinterpret_cast<uint32_t*>(l), cmn[i]);
         atomicMax(reinterpret_cast<uint32_t*>(l + L - 1), cmx[i]);
     }
 }
 
-// Any channel count and alignment (unaligned rates; more than kAnyChannels channels that are no
-// multiple of 64): thread e0 visits elements e0, e0 + S, e0 + 2S, ... with S a
+// Any channel count and alignment (unaligned rates; more than 256 heads with few samples or no
+// multiple of 4): thread e0 visits elements e0, e0 + S, e0 + 2S, ... with S a
 // multiple of nchan, so its channel is fixed.
 __global__ void decay_minmax_kernel(const float* __restrict__ s, long long total, int nchan,
                                     int L, float* lut, int* status) {
@@ -294,13 +304,18 @@ cudaError_t launch_quant_decay(const float* s, long long count, int nchan, int g
     const long long total = count * nchan;
     decay_init_kernel<<<(nchan + 255) / 256, 256, 0, stream>>>(lut, nchan, L);
     // The 16-byte walk where a lane's channels can stay fixed: row decay always (channels a multiple
-    // of 64), heads up to kAnyChannels; codes of up to 16 levels, whose thresholds fit in registers.
+    // of 64), and heads; codes of up to 16 levels, whose thresholds fit in registers.
     // A rate at a time, every thread's extrema went to the few channels by global atomics: call by
     // call from a cold L2, 118 x 256 x 12 rates took 221 us and 256 x 1024 x 1 took 360 us; the walk
     // takes 30 and 28 us (of which 14 us are the call and its four launches).
+    // Above 256 heads the walk needs nchan / gcd(nchan, 1024) blocks, all resident (2 per SM at 16 levels):
+    // heads in fours, at most 255 blocks.  4 levels, calls replayed in a graph: 65536 samples of 1020 heads
+    // 106 us, 264 a rate at a time; 4096 of 260 15 and 32; 1024 of 1000 14.6 and 16.7, of 1020 17.0 and
+    // 16.2; 64 of 1000 12.1 and 9.8, hence the line at 1024 samples.
     const bool aligned = (reinterpret_cast<uintptr_t>(s) & 15) == 0 && (reinterpret_cast<uintptr_t>(codes) & 3) == 0;
     const bool fixed = nchan % 128 == 0 || 128 % nchan == 0;
-    const int lc = fixed || (nchan % 64 != 0 && nchan <= kAnyChannels) ? 32 : nchan % 64 == 0 ? 16 : 0;
+    const bool heads = nchan % 64 != 0 && (nchan <= 256 || (nchan <= kAnyChannels && nchan % 4 == 0 && count >= 1024));
+    const int lc = fixed || heads ? 32 : nchan % 64 == 0 ? 16 : 0;
     const bool any = lc == 32 && !fixed;
     const bool walk = aligned && lc > 0;
     Walk wk = {};
@@ -316,14 +331,17 @@ cudaError_t launch_quant_decay(const float* s, long long count, int nchan, int g
         if (any) turn = nchan / gcd_ll(nchan, 4 * kDecayThreads);
     }
     // resident blocks, a whole number per chunk; fewer when there are not two strips for each lane
-    auto blocks_of = [&](int per_sm) {
+    auto blocks_of = [&](int per_sm, long long most = 1LL << 31) {
         const long long rs = kDecayThreads / lc;
-        const long long want = std::max(1LL, static_cast<long long>(device_sm_count()) * per_sm / wk.chunks);
+        const long long want = std::min(most, std::max(1LL, static_cast<long long>(device_sm_count()) * per_sm / wk.chunks));
         const long long b = std::max(1LL, std::min(want, (wk.strips + rs * 2 - 1) / (rs * 2)));
         return static_cast<unsigned>(wk.chunks * (any ? std::max(turn, b / turn * turn) : b));
     };
     if (walk) {
-#define QS_DM(LC, ANY) decay_minmax_rows_kernel<LC, ANY><<<blocks_of(kMinmaxBlocks), kDecayThreads, 0, stream>>>(s, wk, L, lut, status)
+        // of many heads, each block's extrema are as many atomics: 16 samples to a block at least (4096
+        // samples of 1000 heads, 4 levels: 30 us without this)
+        const long long most = any && nchan > 256 ? std::max(1LL, count / 16) : 1LL << 31;
+#define QS_DM(LC, ANY) decay_minmax_rows_kernel<LC, ANY><<<blocks_of(kMinmaxBlocks, most), kDecayThreads, 0, stream>>>(s, wk, L, lut, status)
         if (any) QS_DM(32, true);
         else if (lc == 32) QS_DM(32, false);
         else QS_DM(16, false);

@@ -47,3 +47,25 @@ def test_quant_decay_rejects_bad_rates(qs, row, H, at, bad):
     with pytest.raises(qs.QstateError):
         qs.qstate_check()
     qs.qstate_check()
+
+
+@pytest.mark.parametrize("H", [260, 300, 516, 1000, 1020])
+@pytest.mark.parametrize("g", [1, 2, 4, 5])
+@pytest.mark.parametrize("B,T,pad", [(1, 1, 0), (1, 1023, 0), (2, 512, 0), (1, 1283, 0), (1, 1024, 1)])
+def test_quant_decay_many_heads(qs, orc, H, g, B, T, pad):
+    """Above 256 heads, in fours and from 1024 samples on: blocks in multiples of H / gcd(H, 1024), up to 255;
+    others a rate at a time."""
+    test_quant_decay_walks(qs, orc, 0, H, 64, g, B, T, pad)
+
+
+@pytest.mark.parametrize("H", [260, 1020])
+@pytest.mark.parametrize("at", [0, -1, 4567])
+def test_quant_decay_many_heads_bad_rate(qs, H, at):
+    cfg = qs.Config(B=1, H=H, dk=128, dv=64, decay_kind=1, unit_kind=1, gate_bits=2)
+    s = torch.rand((1, 1040, H), device="cuda") + 0.1
+    s.view(-1)[at] = -1.0
+    qs.qstate_quant_decay(cfg, s, torch.zeros(s.shape, dtype=torch.uint8, device="cuda"),
+                          torch.zeros(H * 4, device="cuda"), torch.zeros(H * 3, device="cuda"))
+    with pytest.raises(qs.QstateError):
+        qs.qstate_check()
+    qs.qstate_check()
