@@ -16,6 +16,7 @@
  * Parity unpinned: none.  Every function here is pinned by a CPU test against closed forms,
  * printed values of the paper, brute force or an independent formulation.
  */
+#include <float.h>
 #include <math.h>
 #include <stdint.h>
 #include <stdlib.h>
@@ -78,7 +79,7 @@ static float fit_factor(int k) { return (float)((5.0 + (double)k) / 20.0); }
 float orc_expm1_series(float x) {
     if (!(x > 0.0f)) return 0.0f;
     int halvings = 0;
-    while (x > 1.0f) {
+    while (x > 1.0f && x <= FLT_MAX) {   /* an infinite argument: the series is infinite as it is */
         x = x * 0.5f;
         halvings++;
     }

@@ -43,11 +43,12 @@ constexpr int kNullKey = 16 << 24;
 constexpr int kNoKey = 0;
 constexpr int kBins = 128, kBPL = kBins / 32;
 
-// expm1 by its Taylor series (degree 16, Horner), the argument halved while above 1.
+// expm1 by its Taylor series (degree 16, Horner), the argument halved while above 1 (an infinite one
+// cannot be halved; its series is infinite as it is).
 __device__ __noinline__ float expm1_series(float x, const AllocParams& p) {
     if (!(x > 0.0f)) return 0.0f;
     int halvings = 0;
-    while (x > 1.0f) {
+    while (x > 1.0f && x < INFINITY) {
         x = __fmul_rn(x, 0.5f);
         ++halvings;
     }

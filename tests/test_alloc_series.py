@@ -28,3 +28,12 @@ def test_short_series_is_bit_exact(e):
 def test_series_is_the_oracles(orc):
     for x in np.float32([0.12, 0.11, 1e-2, 3e-3, 1e-5]):
         assert np.float32(orc.expm1_series(float(x))) == horner(np.array([x]), 9)[0]
+
+
+@pytest.mark.timeout(60, method="thread")
+def test_series_of_an_infinite_argument(orc):
+    """An erasure statistic that overflowed (|k|^2 beyond FP32's range): the halving must end.  expm1 is
+    infinite, and so from about 89 on."""
+    for x in (np.inf, np.finfo(np.float32).max, 1e30, 200.0):
+        assert orc.expm1_series(float(np.float32(x))) == np.inf
+    assert orc.expm1_series(float("nan")) == 0.0 and orc.expm1_series(float("-inf")) == 0.0

@@ -41,3 +41,26 @@ def test_alloc_launch_rule(qs, orc, shape, stats):
     wref, oref = orc.alloc(co, ms, mr, R)
     assert np.array_equal(widths.cpu().numpy(), wref)
     assert np.array_equal(off.cpu().numpy().view(np.uint32), oref)
+
+
+@pytest.mark.parametrize("shape", [(2, 1, 64, 64, 0, 1), (2, 33, 128, 64, 0, 1), (1, 128, 128, 128, 0, 1), (2, 37, 128, 128, 1, 1)],
+                         ids=lambda s: "x".join(map(str, s)))
+@pytest.mark.parametrize("kind", [0, 2, 6, 7])
+def test_alloc_statistics_beyond_range(qs, orc, shape, kind):
+    """Erasure statistics that overflowed, or are NaN: those units weigh nothing (NaN: as without erasure)."""
+    B, H, dk, dv, head, group = shape
+    kw = dict(B=B, H=H, dk=dk, dv=dv, decay_kind=head, unit_kind=head, group_heads=group, bmin=1, bmax=8, weight_kind=kind)
+    cq, co = qs.Config(bbar_num=3, bbar_den=1, **kw), orc.Cfg(bbar_num=3, **kw)
+    n = B * cq.units
+    rng = np.random.default_rng(n + kind)
+    ms, mr = rng.uniform(0.02, 0.7, n).astype(np.float32), rng.uniform(0, 0.02, n).astype(np.float32)
+    R = np.exp(rng.normal(0, 1, n)).astype(np.float32)
+    for v in (np.inf, -np.inf, np.nan, np.finfo(np.float32).max, 1e20, 89.0, 88.0):
+        mr[rng.choice(n, max(1, n // 50), replace=False)] = v
+    put = lambda a: torch.from_numpy(a).cuda()  # noqa: E731
+    widths, off = put(np.zeros(n, np.uint8)), torch.zeros(B * H, dtype=torch.int32, device="cuda")
+    qs.qstate_alloc_bits(cq, qs.Stats(put(ms), put(mr), put(R)), widths, off)
+    qs.qstate_check()
+    wref, oref = orc.alloc(co, ms, mr, R)
+    assert np.array_equal(widths.cpu().numpy(), wref)
+    assert np.array_equal(off.cpu().numpy().view(np.uint32), oref)
