@@ -87,7 +87,7 @@ __device__ __noinline__ float other_weight(int kind, float ms, float mr, const A
         }
         return __fdiv_rn(1.0f, __fsub_rn(1.0f, pw));
     }
-    if (kind == QSTATE_WEIGHT_NOERASE || mr < 0.0f) mr = 0.0f;
+    if (mr < 0.0f) mr = 0.0f;
     return __fdiv_rn(__fsub_rn(1.0f, ms), __fadd_rn(expm1_series(mr, p), ms));
 }
 
@@ -131,11 +131,11 @@ struct AllocTail {
     int hbytes[1024];                     // payload bytes per head
     int hs, rank, low, left, cnt, ties;   // selection (see below)
     int wties[kThreads / 32];             // tied units per warp
-    int wsum[kThreads / 32];              // sum of widths per warp
+    int wsum[kThreads / 32];              // sum of widths, then of payload bytes, per warp
 };
 
 // UPT consecutive units per thread.  PLAIN: the weights are Eq. 3's (weight_kind OURS) and, for
-// UPT > 1, the arrays aligned for 16-byte loads; otherwise any weight and alignment.
+// UPT > 1, the arrays aligned for 16-byte loads (p.vec); otherwise any weight and alignment.
 template <int UPT, bool PLAIN>
 __global__ void __launch_bounds__(kThreads, 1) alloc_kernel(const __grid_constant__ AllocParams p) {
     extern __shared__ __align__(16) uint8_t smem[];
@@ -163,20 +163,25 @@ __global__ void __launch_bounds__(kThreads, 1) alloc_kernel(const __grid_constan
         //    hit different banks
         float R[UPT], ms[UPT], mr[UPT];
         const bool some = u0 < N;
-        if constexpr (PLAIN && UPT > 1) {
+        if (UPT > 1 && (PLAIN || (p.vec && kind != QSTATE_WEIGHT_SHUFFLE))) {
+            if constexpr (UPT > 1) {
 #pragma unroll
-            for (int k = 0; k < UPT; k += 4) {
-                float4 t = make_float4(0.0f, 0.0f, 0.0f, 0.0f), a = t, b = t;
-                if (some) {
-                    t = *reinterpret_cast<const float4*>(p.range + base + u0 + k);
-                    a = *reinterpret_cast<const float4*>(p.ema_s + base + u0 + k);
-                    b = *reinterpret_cast<const float4*>(p.ema_r + base + u0 + k);
+                for (int k = 0; k < UPT; k += 4) {
+                    float4 t = make_float4(0.0f, 0.0f, 0.0f, 0.0f), a = t, b = t;
+                    if (some) {
+                        t = *reinterpret_cast<const float4*>(p.range + base + u0 + k);
+                        a = *reinterpret_cast<const float4*>(p.ema_s + base + u0 + k);
+                        if (PLAIN || kind != QSTATE_WEIGHT_NOERASE)
+                            b = *reinterpret_cast<const float4*>(p.ema_r + base + u0 + k);
+                    }
+                    R[k] = t.x; R[k + 1] = t.y; R[k + 2] = t.z; R[k + 3] = t.w;
+                    ms[k] = a.x; ms[k + 1] = a.y; ms[k + 2] = a.z; ms[k + 3] = a.w;
+                    mr[k] = b.x; mr[k + 1] = b.y; mr[k + 2] = b.z; mr[k + 3] = b.w;
                 }
-                R[k] = t.x; R[k + 1] = t.y; R[k + 2] = t.z; R[k + 3] = t.w;
-                ms[k] = a.x; ms[k + 1] = a.y; ms[k + 2] = a.z; ms[k + 3] = a.w;
-                mr[k] = b.x; mr[k + 1] = b.y; mr[k + 2] = b.z; mr[k + 3] = b.w;
             }
         } else {
+            // SHUFFLE: the statistics of unit pi(u) (below 2^28 + 2^14: 32 bits)
+            int pi = !PLAIN && kind == QSTATE_WEIGHT_SHUFFLE ? (p.shuf_a * u0 + p.shuf_b) % N : 0;
 #pragma unroll
             for (int k = 0; k < UPT; ++k) {
                 const int u = u0 + k;
@@ -184,11 +189,14 @@ __global__ void __launch_bounds__(kThreads, 1) alloc_kernel(const __grid_constan
                 ms[k] = 1.0f;
                 if (u < N) {
                     int us = u;
-                    if (!PLAIN && kind == QSTATE_WEIGHT_SHUFFLE)   // the statistics of unit pi(u)
-                        us = static_cast<int>((static_cast<long long>(p.shuf_a) * u + p.shuf_b) % N);
+                    if (!PLAIN && kind == QSTATE_WEIGHT_SHUFFLE) {
+                        us = pi;
+                        pi += p.shuf_a;
+                        if (pi >= N) pi -= N;
+                    }
                     if (p.unit_row) R[k] = p.range[base + u];
                     ms[k] = p.ema_s[base + us];
-                    mr[k] = p.ema_r[base + us];
+                    if (PLAIN || kind != QSTATE_WEIGHT_NOERASE) mr[k] = p.ema_r[base + us];
                 }
             }
         }
@@ -239,8 +247,10 @@ __global__ void __launch_bounds__(kThreads, 1) alloc_kernel(const __grid_constan
             }
         }
         float c[UPT];
-        {
-            bool rare = !PLAIN && kind != QSTATE_WEIGHT_OURS;
+        // Gamma_hat (Eq. 3), for the weights that have it
+        if (PLAIN || kind == QSTATE_WEIGHT_OURS || kind == QSTATE_WEIGHT_GAMMA_RAW || kind == QSTATE_WEIGHT_NOERASE ||
+            kind == QSTATE_WEIGHT_SHUFFLE) {
+            bool rare = false;
 #pragma unroll
             for (int k = 0; k < UPT; ++k) rare |= !(mr[k] < kShortSeries) || mr[k] < 0.0f;
             // (-0 and 0 give expm1 = +-0, which adds nothing to m_s)
@@ -250,9 +260,12 @@ __global__ void __launch_bounds__(kThreads, 1) alloc_kernel(const __grid_constan
             if (rare) {
 #pragma unroll
                 for (int k = 0; k < UPT; ++k)
-                    if ((!PLAIN && kind != QSTATE_WEIGHT_OURS) || !(mr[k] < kShortSeries) || mr[k] < 0.0f)
-                        c[k] = other_weight(kind, ms[k], mr[k], p);
+                    if (!(mr[k] < kShortSeries) || mr[k] < 0.0f) c[k] = other_weight(kind, ms[k], mr[k], p);
             }
+        } else {
+            const bool flat = kind == QSTATE_WEIGHT_RANGE || kind == QSTATE_WEIGHT_NRANGE;
+#pragma unroll
+            for (int k = 0; k < UPT; ++k) c[k] = flat ? 1.0f : other_weight(kind, ms[k], mr[k], p);
         }
         if (p.unit_row) {
             __syncthreads();
@@ -266,10 +279,6 @@ __global__ void __launch_bounds__(kThreads, 1) alloc_kernel(const __grid_constan
                 c[k] = alone ? f : __fmul_rn(c[k], f);
             }
         } else {
-            if (!PLAIN && (kind == QSTATE_WEIGHT_RANGE || kind == QSTATE_WEIGHT_NRANGE)) {
-#pragma unroll
-                for (int k = 0; k < UPT; ++k) c[k] = 1.0f;
-            }
             __syncthreads();   // the histogram is zero
         }
 
@@ -410,12 +419,14 @@ __global__ void __launch_bounds__(kThreads, 1) alloc_kernel(const __grid_constan
 
     // 6. widths out; head offsets: exclusive prefix sum of the heads' payload bytes (row unit: the
     //    dk / UPT consecutive lanes of a head sum its widths)
-    if constexpr (PLAIN && UPT > 1) {
-        if (u0 < N)
+    if (UPT > 1 && (PLAIN || p.vec)) {
+        if constexpr (UPT > 1) {
+            if (u0 < N)
 #pragma unroll
-            for (int k = 0; k < UPT; k += 4)
-                *reinterpret_cast<uint32_t*>(p.widths + base + u0 + k) =
-                    static_cast<uint32_t>(w[k] | (w[k + 1] << 8) | (w[k + 2] << 16) | (w[k + 3] << 24));
+                for (int k = 0; k < UPT; k += 4)
+                    *reinterpret_cast<uint32_t*>(p.widths + base + u0 + k) =
+                        static_cast<uint32_t>(w[k] | (w[k + 1] << 8) | (w[k + 2] << 16) | (w[k + 3] << 24));
+        }
     } else {
 #pragma unroll
         for (int k = 0; k < UPT; ++k)
@@ -446,7 +457,10 @@ __global__ void __launch_bounds__(kThreads, 1) alloc_kernel(const __grid_constan
             if (u0 + k < N) sm.hbytes[u0 + k] = w[k] * p.dk * p.dv / 8;
     }
     __syncthreads();
-    if (warp == 0) {
+    // 32 heads at a time by one warp, or, of many, 32 by each warp (1024 heads, head unit: 7.1 us a
+    // launch by one warp, 3.6; 256: 3.7 and 2.9; 65: 3.0 and 2.8)
+    if (p.H <= 64) {
+        if (warp != 0) return;
         int carry = 0;
 #pragma unroll 1
         for (int h0 = 0; h0 < p.H; h0 += 32) {
@@ -457,6 +471,13 @@ __global__ void __launch_bounds__(kThreads, 1) alloc_kernel(const __grid_constan
                 p.head_off[static_cast<size_t>(blockIdx.x) * p.H + h] = static_cast<uint32_t>(carry + incl - v);
             carry += __shfl_sync(kFull, incl, 31);
         }
+    } else {
+        const int v = tid < p.H ? sm.hbytes[tid] : 0;
+        const int incl = warp_prefix(v, lane);
+        if (lane == 31) sm.wsum[warp] = incl;
+        __syncthreads();
+        const int carry = __reduce_add_sync(kFull, lane < warp ? sm.wsum[lane] : 0);
+        if (tid < p.H) p.head_off[static_cast<size_t>(blockIdx.x) * p.H + tid] = static_cast<uint32_t>(carry + incl - v);
     }
 }
 
@@ -482,10 +503,18 @@ cudaError_t launch_alloc(const AllocParams& p_in, cudaStream_t stream) {
     auto aligned = [](const void* q, uintptr_t n) { return (reinterpret_cast<uintptr_t>(q) & (n - 1)) == 0; };
     const bool ours = p.uniform || p.weight_kind == QSTATE_WEIGHT_OURS;
     // row unit: N is a multiple of 64, so every batch element is aligned as the arrays are
-    const bool plain = ours && p.unit_row && aligned(p.widths, 4) &&
-                       (p.uniform || (aligned(p.ema_s, 16) && aligned(p.ema_r, 16) && aligned(p.range, 16)));
+    p.vec = p.unit_row && aligned(p.widths, 4) &&
+                    (p.uniform || (aligned(p.ema_s, 16) && aligned(p.ema_r, 16) && aligned(p.range, 16)))
+                ? 1 : 0;
     if (p.units <= 1024) return ours ? launch_alloc_t<1, true>(p, stream) : launch_alloc_t<1, false>(p, stream);
-    if (!plain) return p.units <= 4096 ? launch_alloc_t<4, false>(p, stream) : launch_alloc_t<16, false>(p, stream);
+    // Other weights and alignments: 8 units per thread up to 8192 units as below.  One batch element, range
+    // weights: 8192 units 9.9 us, 16384 19.5 us (38 and 66 us with 16 units per thread at 8192, the
+    // decay part evaluated for every weight kind by the full series, and 4-byte loads); shuffled decay weights
+    // 13.9 and 34.9 us (38.8 and 70); statistics off 16 bytes 13.9 and 35 us (20.1 and 36).
+    if (!ours || !p.vec)
+        return p.units <= 4096   ? launch_alloc_t<4, false>(p, stream)
+               : p.units <= 8192 ? launch_alloc_t<8, false>(p, stream)
+                                 : launch_alloc_t<16, false>(p, stream);
     // Units per thread: as few as 1024 threads allow, for the latency of a launch with few batch
     // elements (4096 units: 6.1 us with 4 per thread, 6.5 us with 8).  Launches of many run beside
     // write-backs, whose CTAs they displace: 512 threads there (KDA decode, 4096 units, 4 x 64

@@ -83,6 +83,7 @@ struct AllocParams {
     int shuf_a, shuf_b;   // shuffled-decay bijection u -> (shuf_a u + shuf_b) mod units
     int ngroups, gshift, above_min;   // set by launch_alloc: normalisation groups, log2 of their
                                       // size (-1: no power of two), total - units bmin
+    int vec;                          // set by launch_alloc: arrays aligned for 16-byte loads
     const float* ema_s;
     const float* ema_r;
     const float* range;

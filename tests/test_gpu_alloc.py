@@ -64,3 +64,27 @@ def test_alloc_statistics_beyond_range(qs, orc, shape, kind):
     wref, oref = orc.alloc(co, ms, mr, R)
     assert np.array_equal(widths.cpu().numpy(), wref)
     assert np.array_equal(off.cpu().numpy().view(np.uint32), oref)
+
+
+@pytest.mark.parametrize("shape", [(2, 33, 128, 64, 0, 1), (1, 65, 64, 64, 0, 5), (1, 65, 128, 128, 0, 5), (1, 128, 128, 128, 0, 1),
+                                   (2, 65, 128, 128, 1, 1), (1, 1024, 64, 64, 1, 1)], ids=lambda s: "x".join(map(str, s)))
+@pytest.mark.parametrize("kind", [1, 3, 4, 5, 6, 7, 8])
+@pytest.mark.parametrize("pad", [0, 1])
+def test_alloc_other_weights(qs, orc, shape, kind, pad):
+    """The other weights at every number of units per thread, aligned and not; heads above 64, whose offsets
+    are summed by a warp for each 32."""
+    B, H, dk, dv, head, group = shape
+    kw = dict(B=B, H=H, dk=dk, dv=dv, decay_kind=head, unit_kind=head, group_heads=group, bmin=1, bmax=8,
+              weight_kind=kind, C=13)
+    cq, co = qs.Config(bbar_num=3, bbar_den=1, **kw), orc.Cfg(bbar_num=3, **kw)
+    n = B * cq.units
+    rng = np.random.default_rng(n + kind)
+    ms, mr = rng.uniform(0.02, 0.7, n).astype(np.float32), rng.uniform(0, 0.3, n).astype(np.float32)
+    R = np.exp(rng.normal(0, 1, n)).astype(np.float32)
+    put = lambda a: torch.from_numpy(np.concatenate([np.zeros(pad, a.dtype), a])).cuda()[pad:]  # noqa: E731
+    widths, off = put(np.zeros(n, np.uint8)), torch.zeros(B * H, dtype=torch.int32, device="cuda")
+    qs.qstate_alloc_bits(cq, qs.Stats(put(ms), put(mr), put(R)), widths, off)
+    qs.qstate_check()
+    wref, oref = orc.alloc(co, ms, mr, R)
+    assert np.array_equal(widths.cpu().numpy(), wref)
+    assert np.array_equal(off.cpu().numpy().view(np.uint32), oref)
