@@ -6,7 +6,8 @@
 // The value columns of a head are independent (p_j, u_j, o_j and column j of the state need only
 // column j and the token's row vectors), so a CTA of 4 warps takes 64 columns of a head and a warp
 // 16 of them over all key rows, with no exchange between warps.  Lane (rg, cg) = (lane / 2,
-// lane % 2) owns RL = dk / 16 rows x 8 columns.  Per token it reads its rows' d, k and q from
+// lane % 2) owns RL = dk / 16 rows x 8 columns (two runs of 4, so that a lane pair's 16-byte accesses
+// fill 32-byte sectors).  Per token it reads its rows' d, k and q from
 // shared memory (24 bytes per row for 8 columns x 4 multiply-adds: with 4 columns per lane the
 // shared-memory path would be as busy as the FMA pipe), decays, and forms p = a^T S' and r = q^T S'
 // over its rows with row pairs as packed operands (d, k and q come from memory as pairs); 15
@@ -18,6 +19,10 @@
 // them, the chain of each token's sums, which the 16 warps per SM do not quite hide.  16 x 32 heads
 // of 128 x 128, 32 tokens: 74 us; 463 us with a launch per token, each reading and writing the
 // state (67 MB).
+// A call of one token is its state's trip through memory: 16 x 32 heads of 128 x 128 16.6 us from
+// HBM (4.0 TB/s; 18.3 us with 8 neighbouring columns per lane, whose accesses took half a sector each)
+// and 14.1 us from L2 (16.8 us), bound by the L1's lookups, as a warp's 16 columns are 64 bytes of a row; a
+// kernel whose warps hold whole rows takes 16.4 and 11.4 us there, and 26.7 us for 4 tokens (19 us here).
 #include "qs_common.cuh"
 
 namespace qs {
@@ -85,7 +90,8 @@ __global__ void __launch_bounds__(kFpThreads, 4) scan_fp32_kernel(const __grid_c
     // 64 values without gaps, on all banks)
     const int i0 = (lane >> 1) * 4;
     auto row = [](int r) { return (r / 4) * 64 + r % 4; };   // + i0
-    const int j0 = c0 + 16 * warp + 8 * (lane & 1);   // and first column
+    // and columns: 4 from j0 on and 4 from j0 + 8 on, so that a lane pair's 16-byte accesses fill sectors
+    const int j0 = c0 + 16 * warp + 4 * (lane & 1);
 
     auto issue = [&](St& S, int t0) {
         const int nt = min(kTB, p.t_end - t0);
@@ -137,12 +143,12 @@ __global__ void __launch_bounds__(kFpThreads, 4) scan_fp32_kernel(const __grid_c
         float t[8];
         if (vec & 2) {
             const float4 lo = *reinterpret_cast<const float4*>(src + row(r) * dv);
-            const float4 hi = *reinterpret_cast<const float4*>(src + row(r) * dv + 4);
+            const float4 hi = *reinterpret_cast<const float4*>(src + row(r) * dv + 8);
             t[0] = lo.x; t[1] = lo.y; t[2] = lo.z; t[3] = lo.w;
             t[4] = hi.x; t[5] = hi.y; t[6] = hi.z; t[7] = hi.w;
         } else {
 #pragma unroll
-            for (int c = 0; c < 8; ++c) t[c] = src[row(r) * dv + c];
+            for (int c = 0; c < 8; ++c) t[c] = src[row(r) * dv + (c & 3) + 2 * (c & 4)];
         }
 #pragma unroll
         for (int c = 0; c < 8; ++c) {
@@ -234,7 +240,7 @@ __global__ void __launch_bounds__(kFpThreads, 4) scan_fp32_kernel(const __grid_c
             halve<4>(s, lane, 4);
             halve<2>(s, lane, 2);
             if constexpr (ERASE == kEraseNone) s[0] += __shfl_xor_sync(kFull, s[0], 16);
-            const int jl = 8 * (lane & 1) + ((lane & 8) ? 4 : 0) + ((lane & 4) ? 2 : 0) + ((lane & 2) ? 1 : 0);
+            const int jl = 4 * (lane & 1) + ((lane & 8) ? 8 : 0) + ((lane & 4) ? 2 : 0) + ((lane & 2) ? 1 : 0);
             const int jc = 16 * warp + jl;   // the lane's column within the CTA's
             const float vj = S.v[t][jc];
             // u = w o v - p (w = beta 1, p = beta k^T S' for the delta rule; a = 0, w = 1 without)
@@ -249,8 +255,8 @@ __global__ void __launch_bounds__(kFpThreads, 4) scan_fp32_kernel(const __grid_c
             __syncwarp();
             if (lane >= 16)   // o = S^T q = r + u (k . q)
                 p.o[((static_cast<size_t>(b) * p.T + t0 + t) * p.H + h) * dv + c0 + jc] = fmaf(u, kq, s[0]);
-            const float4 ua = *reinterpret_cast<const float4*>(&sm.u[warp][8 * (lane & 1)]);
-            const float4 ub = *reinterpret_cast<const float4*>(&sm.u[warp][8 * (lane & 1) + 4]);
+            const float4 ua = *reinterpret_cast<const float4*>(&sm.u[warp][4 * (lane & 1)]);
+            const float4 ub = *reinterpret_cast<const float4*>(&sm.u[warp][4 * (lane & 1) + 8]);
             const float us[8] = {ua.x, ua.y, ua.z, ua.w, ub.x, ub.y, ub.z, ub.w};
 #pragma unroll
             for (int m = 0; m < RL / 2; m += 2) {
@@ -273,10 +279,10 @@ __global__ void __launch_bounds__(kFpThreads, 4) scan_fp32_kernel(const __grid_c
         for (int c = 0; c < 8; ++c) t[c] = r & 1 ? x[r / 2][c].y : x[r / 2][c].x;
         if (vec & 2) {
             *reinterpret_cast<float4*>(dst + row(r) * dv) = make_float4(t[0], t[1], t[2], t[3]);
-            *reinterpret_cast<float4*>(dst + row(r) * dv + 4) = make_float4(t[4], t[5], t[6], t[7]);
+            *reinterpret_cast<float4*>(dst + row(r) * dv + 8) = make_float4(t[4], t[5], t[6], t[7]);
         } else {
 #pragma unroll
-            for (int c = 0; c < 8; ++c) dst[row(r) * dv + c] = t[c];
+            for (int c = 0; c < 8; ++c) dst[row(r) * dv + (c & 3) + 2 * (c & 4)] = t[c];
         }
     }
 }
