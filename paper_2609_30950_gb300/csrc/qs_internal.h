@@ -116,8 +116,6 @@ cudaError_t launch_chained(void (*kern)(P...), int grid, int threads, size_t sme
 }
 
 // launchers (return cudaError_t of the launch)
-cudaError_t launch_step(const qstate_cfg& cfg, int src_packed, int dst_packed,
-                        const StepParams& p, cudaStream_t stream);
 cudaError_t launch_scan_fp32(int dk, int dv, const StepParams& p, cudaStream_t stream);
 cudaError_t launch_alloc(const AllocParams& p, cudaStream_t stream);
 cudaError_t launch_quant_decay(const float* s, long long count, int nchan, int g,

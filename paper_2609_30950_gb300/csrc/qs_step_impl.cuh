@@ -1,6 +1,7 @@
-// qs_step_impl.cuh -- write-back kernel of libqstate for the row allocation unit where buffers are not
-// 16-byte aligned (sm_103a; aligned ones take qs_wb_row.cuh), and the dispatch of write-back, pack and
-// unpack by state shape and unit.
+// qs_step_impl.cuh -- write-back kernel of libqstate for the row allocation unit where token inputs,
+// metadata or statistics are not 16-byte aligned (sm_103a; aligned ones take qs_wb_row.cuh; payloads
+// are aligned to 16 bytes at dv = 128, 8 at dv = 64, for every kernel), and the dispatch of write-back,
+// pack and unpack by state shape and unit.
 //
 // One CTA per (batch element, head), 8 warps.  Warp w owns key rows [w*RPW, (w+1)*RPW); lane
 // l owns value columns [l*CPL, (l+1)*CPL) of each of them, so one row is handled by one warp
@@ -44,7 +45,7 @@ struct alignas(16) StepSmem {
     float rowR[DK], rowM[DK], rowD[DK], rowInv[DK];
     float fitf[kNFit];                    // f_k = (5 + k) / 20
     float inv_n[17];                      // 1 / (2^(w-1) - 1), w = 2..16
-    float wsum[4][NW];                    // per-warp partial k.q, |k|^2, a.k, |a|^2
+    float wsum[DK / 32];                  // per-warp partial k.q
     int off_in[DK + 1], off_out[DK + 1];  // row byte offsets inside the head (+ total)
     uint16_t out_scale[NSG];
     uint8_t out_fidx[NSG];
@@ -240,15 +241,7 @@ __global__ void __launch_bounds__(256, 2) step_kernel(const StepParams p) {
                 }
             }
             const float kq = warp_sum(kk * qq);
-            const float k2 = warp_sum(kk * kk);
-            const float ak = warp_sum(ai * kk);
-            const float aa = warp_sum(ai * ai);
-            if (lane == 0) {
-                sm.wsum[0][warp] = kq;
-                sm.wsum[1][warp] = k2;
-                sm.wsum[2][warp] = ak;
-                sm.wsum[3][warp] = aa;
-            }
+            if (lane == 0) sm.wsum[warp] = kq;
         }
         if (tid < DV) {
             sm.v[tid] = __ldg(p.v + tok * DV + tid);
@@ -305,7 +298,7 @@ __global__ void __launch_bounds__(256, 2) step_kernel(const StepParams p) {
                 Rr += sm.red[1][w][j];
             }
 #pragma unroll
-            for (int w = 0; w < DK / 32; ++w) kq += sm.wsum[0][w];
+            for (int w = 0; w < DK / 32; ++w) kq += sm.wsum[w];
             const float vj = sm.v[j];
             // S = S' - k (a^T S') + k (w o v)^T:  u = beta v - p (delta rule), u = v (no erase)
             const float wj = p.general ? sm.gw[j] : beta;

@@ -86,3 +86,18 @@ def test_dense_state(qs, dk, dv, head, pad):
         got.append((st.payload, st.scales, st.fidx, view.clone()))
     for a, b in zip(*got):
         assert torch.equal(a, b)
+
+
+ARRAYS = {"token inputs": ("q", "k", "v", "s", "s_code", "beta", "a", "w"), "metadata": ("scales", "widths", "fidx"),
+          "statistics": ("ema_s", "ema_r", "range")}
+
+
+@pytest.mark.parametrize("dk,dv", [(128, 128), (128, 64), (64, 64)])
+@pytest.mark.parametrize("name,gate_bits", [("kda_decode", 0), ("kda_decode", 2), ("kda_decode", 4), ("mamba2_decode", 0),
+                                            ("kda_general", 0), ("gdn_decode", 0), ("gdn_decode", 3), ("gdn_general", 0)])
+@pytest.mark.parametrize("arrays,C,fit_every", [("token inputs", 1, 1), ("metadata", 3, 1), ("statistics", 4, 3)])
+def test_write_back(qs, orc, dk, dv, name, gate_bits, arrays, C, fit_every):
+    """Everything but the payload off its boundary, row unit and head unit."""
+    w = synth.scaled(WORKLOADS[name], B=2, H=4, T=9, C=C, dk=dk, dv=dv, group_heads=2 if "mamba" in name else 1,
+                     gate_bits=gate_bits)
+    _lockstep(Shifted(qs, *ARRAYS[arrays]), orc, w, log_decay=gate_bits > 0, fit_every=fit_every)
