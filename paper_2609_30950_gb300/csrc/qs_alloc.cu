@@ -516,10 +516,14 @@ cudaError_t launch_alloc(const AllocParams& p_in, cudaStream_t stream) {
                : p.units <= 8192 ? launch_alloc_t<8, false>(p, stream)
                                  : launch_alloc_t<16, false>(p, stream);
     // Units per thread: as few as 1024 threads allow, for the latency of a launch with few batch
-    // elements (4096 units: 6.1 us with 4 per thread, 6.5 us with 8).  Launches of many run beside
-    // write-backs, whose CTAs they displace: 512 threads there (KDA decode, 4096 units, 4 x 64
-    // batch elements: 378 us per token with 8 per thread, 386 us with 4); at 8192 units that would
-    // be 16 per thread, which cost more than it gave (Mamba-2: 211 against 210 us).
+    // elements (4096 units: 6.9 us with 4 per thread, 7.4 us with 8).  Launches of many run beside
+    // write-backs, whose CTAs they displace: 512 threads there.  KDA decode in four partitions, per token
+    // with 4 and with 8 units per thread: partitions of 2 batch elements of 4096 units 27.4 and 27.5 us, of 8
+    // 51.2 and 48.7, of 16 97.0 and 96.1, of 32 183.9 and 178.1, of 64 355.8 and 344.4; of 3072 units 25.4 and
+    // 26.2, 40.8 and 39.4, 76.6 and 77.2, 140.0 and 136.7, 273.5 and 262.6.  In one chain, where nothing runs
+    // beside them: 16 batch elements 35.4 and 35.7, 32 61.0 and 61.2, 64 100.3 and 100.8.  Hence 8 from the
+    // size on at which it gains for both.  At 8192 units the same would be 16 per thread,
+    // which cost more than it gave (Mamba-2: 211 against 210 us).
     if (p.units <= 4096) return p.units > 2048 && p.B >= 32 ? launch_alloc_t<8, true>(p, stream) : launch_alloc_t<4, true>(p, stream);
     if (p.units <= 8192) return launch_alloc_t<8, true>(p, stream);
     return launch_alloc_t<16, true>(p, stream);

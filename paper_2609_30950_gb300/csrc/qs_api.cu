@@ -459,11 +459,15 @@ ScanArrays slice(const qstate_cfg* c, const qstate_buf* ping, const qstate_buf* 
     return a;
 }
 
-// Partitions of a scan: the requested number, else the count measured best on GB300 for the
-// benchmark layer shapes (token form 4: 6 % per token at KDA decode, 24 % at Gated DeltaNet;
-// chunked form 2: 10 % at KDA prefill, where 3 or 4 split its 16 batch elements less evenly over
-// the one-CTA-per-SM launches); at most one per batch element, and fewer where a partition would
-// start off a 16-byte boundary in any array.
+// Partitions of a scan: the requested number, else 4 for the token form and 2 for the chunked form; at
+// most one per batch element, and fewer where a partition would start off a 16-byte boundary in any
+// array.  Microseconds per write-back at 1 / 2 / 3 / 4 / 8 partitions: KDA decode of 256 x 32 heads 361.9 / 347.1
+// / 342.6 / 344.1 / 350.5, Gated DeltaNet of 64 x 16 48.8 / 39.6 / 41.2 / 37.7 / 37.8 and of 256 x 16 154.3 /
+// 129.9 / 129.8 / 129.6 / 129.6, Mamba-2 of 128 x 64 200.1 / 204.2 / 203.9 / 200.1 / 206.8, KDA prefill of 16 x 32
+// token by token 207.6 / 180.9 / 178.9 / 182.0 / 184.3, chunked 131.9 / 116.5 / 131.0 / 120.5 / 122.7 (3 and 4
+// split 16 batch elements less evenly over the one-CTA-per-SM launches).  Batches that do not fill the SMs
+// once are faster in one chain, whose launches begin early (KDA decode of 16 x 16 heads 20.8 / 23.4 / 25.9 / 25.3 /
+// 37.9, chunked prefill of 4 x 32 40.1 / 45.1 / 47.1 / 47.3 / 47.2): a caller can ask for it.
 int scan_parts(const qstate_cfg* c, const qstate_inputs* x, const qstate_stats* st) {
     int G = g_scan_parts.load();
     if (G <= 0) G = c->interval_form == QSTATE_FORM_CHUNK ? 2 : 4;
