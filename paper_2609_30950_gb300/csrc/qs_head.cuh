@@ -476,8 +476,8 @@ cudaError_t launch_head_t(const qstate_cfg& cfg, const StepParams& p, cudaStream
 // CTAs per SM.  134 x 46 heads of 128 x 64, 4 bits: 86 -> 50 us.  A dense state that is not 16-byte aligned:
 // every 32nd (16th) column to a lane, whose 4-byte stores then have no gaps (512 heads
 // of 128 x 64, 4 bits: 6.0 us; 9.2 with four consecutive columns, 7.2 by the write-back's lanes).
-template <int DK, int DV>
-__global__ void __launch_bounds__(256, 6) unpack_head_kernel(const __grid_constant__ StepParams p, bool vec) {
+template <int DK, int DV, bool VEC>
+__global__ void __launch_bounds__(256, 6) unpack_head_kernel(const __grid_constant__ StepParams p) {
     extern __shared__ __align__(16) uint8_t smem_raw[];
     using Vec = typename std::conditional<DV == 128, uint4, uint2>::type;
     constexpr int NB = DK / 32, WPB = 8 / NB;   // row blocks, and warps in each
@@ -492,7 +492,7 @@ __global__ void __launch_bounds__(256, 6) unpack_head_kernel(const __grid_consta
     const size_t gbase = static_cast<size_t>(g) * NB * DV + static_cast<size_t>(blk) * DV;
     uint16_t sc[4];
 #pragma unroll
-    for (int c = 0; c < 4; ++c) sc[c] = p.in_scales[gbase + (vec ? cl * 4 + c : cl + c * CW)];
+    for (int c = 0; c < 4; ++c) sc[c] = p.in_scales[gbase + (VEC ? cl * 4 + c : cl + c * CW)];
     if (w > 16 || off % static_cast<int>(sizeof(Vec)) != 0 || off + bytes > p.region_bytes || bytes > p.stage_bytes) {
         if (tid == 0) raise_status(p.status, QS_DEV_LAYOUT);   // the whole CTA: nothing has been written
         return;
@@ -514,7 +514,7 @@ __global__ void __launch_bounds__(256, 6) unpack_head_kernel(const __grid_consta
     const int r0 = 32 * blk + (warp % WPB) * RS + half;
     const uint32_t* words = reinterpret_cast<const uint32_t*>(smem_raw) + r0 * rowwords;
     float* dst = p.dense_out + (static_cast<size_t>(g) * DK + r0) * DV;
-    if (!vec) {
+    if constexpr (!VEC) {
 #pragma unroll 2
         for (int r = 0; r < 32; r += WPB * RS) {
 #pragma unroll
@@ -548,9 +548,11 @@ cudaError_t launch_unpack_head_t(const qstate_cfg& cfg, const StepParams& p, cud
     StepParams q = p;
     q.stage_bytes = DK * DV * cfg.bmax / 8;
     const int smem = q.stage_bytes + 16;   // the last lane reads up to 8 bytes past the head's rows
-    cudaError_t e = cudaFuncSetAttribute(unpack_head_kernel<DK, DV>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    const bool vec = (reinterpret_cast<uintptr_t>(p.dense_out) & 15) == 0;
+    auto kern = vec ? unpack_head_kernel<DK, DV, true> : unpack_head_kernel<DK, DV, false>;
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
-    unpack_head_kernel<DK, DV><<<cfg.B * cfg.H, 256, smem, stream>>>(q, (reinterpret_cast<uintptr_t>(p.dense_out) & 15) == 0);
+    kern<<<cfg.B * cfg.H, 256, smem, stream>>>(q);
     return cudaGetLastError();
 }
 

@@ -29,9 +29,9 @@ struct alignas(16) PackSmem {
     int flag, next;
 };
 
-// align: the dense state's alignment, 16, 8 or 4 bytes.
-template <int DK, int DV>
-__global__ void __launch_bounds__(128, 4) pack_row_kernel(const __grid_constant__ StepParams p, int align) {
+// The dense state's alignment: 4 bytes with BY4, else vec: 16 (else 8).
+template <int DK, int DV, bool BY4>
+__global__ void __launch_bounds__(128, 4) pack_row_kernel(const __grid_constant__ StepParams p, bool vec) {
     using RQ = RowQuant<DV>;
     constexpr int TPR = RQ::TPR, RPB = RQ::RPB, NB = DK / RPB, NW = PackSmem<DK, DV>::NW;
     __shared__ PackSmem<DK, DV> sm;
@@ -96,16 +96,16 @@ __global__ void __launch_bounds__(128, 4) pack_row_kernel(const __grid_constant_
             const float* src = p.dense_in + (rb + i) * DV + 32 * q;
 #pragma unroll
             for (int c = 0; c < 8; ++c) {
-                if (align == 16) {
+                if constexpr (BY4) {
+                    xv[2 * c] = make_float2(src[4 * c], src[4 * c + 1]);
+                    xv[2 * c + 1] = make_float2(src[4 * c + 2], src[4 * c + 3]);
+                } else if (vec) {
                     const float4 v = __ldcs(reinterpret_cast<const float4*>(src + 4 * c));
                     xv[2 * c] = make_float2(v.x, v.y);
                     xv[2 * c + 1] = make_float2(v.z, v.w);
-                } else if (align == 8) {
+                } else {
                     xv[2 * c] = *reinterpret_cast<const float2*>(src + 4 * c);
                     xv[2 * c + 1] = *reinterpret_cast<const float2*>(src + 4 * c + 2);
-                } else {
-                    xv[2 * c] = make_float2(src[4 * c], src[4 * c + 1]);
-                    xv[2 * c + 1] = make_float2(src[4 * c + 2], src[4 * c + 3]);
                 }
             }
         } else {
@@ -161,7 +161,8 @@ cudaError_t launch_pack_row_t(const qstate_cfg& cfg, const StepParams& p, cudaSt
     StepParams q = p;
     q.stage_bytes = DK * DV * cfg.bmax / 8;
     const uintptr_t at = reinterpret_cast<uintptr_t>(p.dense_in);
-    pack_row_kernel<DK, DV><<<cfg.B * cfg.H, 128, 0, stream>>>(q, at % 16 == 0 ? 16 : at % 8 == 0 ? 8 : 4);
+    auto kern = at % 8 == 0 ? pack_row_kernel<DK, DV, false> : pack_row_kernel<DK, DV, true>;
+    kern<<<cfg.B * cfg.H, 128, 0, stream>>>(q, at % 16 == 0);
     return cudaGetLastError();
 }
 
@@ -183,8 +184,9 @@ struct alignas(16) UnpackSmem {
     int total, flag, pad[2];
 };
 
-template <int DK, int DV>
-__global__ void __launch_bounds__(256, 6) unpack_row_kernel(const __grid_constant__ StepParams p, bool vec) {
+// VEC: the dense state is 16-byte aligned.
+template <int DK, int DV, bool VEC>
+__global__ void __launch_bounds__(256, 6) unpack_row_kernel(const __grid_constant__ StepParams p) {
     extern __shared__ __align__(16) uint8_t smem_raw[];
     UnpackSmem<DK, DV>& sm = *reinterpret_cast<UnpackSmem<DK, DV>*>(smem_raw);
     uint8_t* pay = smem_raw + sizeof(UnpackSmem<DK, DV>);
@@ -243,7 +245,7 @@ __global__ void __launch_bounds__(256, 6) unpack_row_kernel(const __grid_constan
     }
     constexpr int RS = 128 / DV;   // rows that a warp decodes at once
     const int half = lane / (32 / RS), cl = lane % (32 / RS);
-    if (!vec) {
+    if constexpr (!VEC) {
 #pragma unroll 2
         for (int r = warp * RS + half; r < DK; r += 8 * RS) {
             const float4 dq = sm.deq[r];
@@ -285,9 +287,11 @@ cudaError_t launch_unpack_row_t(const qstate_cfg& cfg, const StepParams& p, cuda
     StepParams q = p;
     q.stage_bytes = DK * DV * cfg.bmax / 8;
     const int smem = static_cast<int>(sizeof(UnpackSmem<DK, DV>)) + q.stage_bytes + 16;   // 12 readable bytes
-    cudaError_t e = cudaFuncSetAttribute(unpack_row_kernel<DK, DV>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    const bool vec = (reinterpret_cast<uintptr_t>(p.dense_out) & 15) == 0;
+    auto kern = vec ? unpack_row_kernel<DK, DV, true> : unpack_row_kernel<DK, DV, false>;
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
-    unpack_row_kernel<DK, DV><<<cfg.B * cfg.H, 256, smem, stream>>>(q, (reinterpret_cast<uintptr_t>(p.dense_out) & 15) == 0);
+    kern<<<cfg.B * cfg.H, 256, smem, stream>>>(q);
     return cudaGetLastError();
 }
 
