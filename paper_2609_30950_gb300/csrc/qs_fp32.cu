@@ -15,7 +15,7 @@
 // shared memory.  The inputs of 8 tokens are copied ahead with cp.async while the 8 before them
 // run; the rates become decays in place.  Two CTA barriers per 8 tokens.
 //
-// What bounds it: 4 FMA-pipe operations per element and token (the pipe is 53 % busy) and, between
+// What bounds it: 4 FMA-pipe operations per element and token (the pipe is 54 % busy) and, between
 // them, the chain of each token's sums, which the 16 warps per SM do not quite hide.  16 x 32 heads
 // of 128 x 128, 32 tokens: 74 us; 463 us with a launch per token, each reading and writing the
 // state (67 MB).

@@ -12,8 +12,8 @@ namespace qs {
 // loads each lane's 32 consecutive values of its row straight from the dense state, and quantises
 // and stores them without any exchange beyond the row's TPR lanes.  16 warps per SM: the loads of
 // some hide behind the searches of the others.
-// What bounds it: the search's FP32 work (about 36 lane-instructions per element), ahead of HBM
-// (64 KB read per head).  64 x 32 heads of 128 x 128, 4 bits: 78 us (151 MB, 1.9 TB/s); 214 us with all
+// What bounds it: the search's FP32 work (47 lane-instructions per element in all; issue 59 %, FMA pipe
+// 56 % of the time, the loads' latency next), ahead of HBM (64 KB read per head).  64 x 32 heads of 128 x 128, 4 bits: 78 us (151 MB, 1.9 TB/s); 214 us with all
 // 16 candidates of every row in scalar arithmetic, a row spread over a warp.  Results are those of that
 // arithmetic bit for bit (each product and sum of a code rounded by itself, near ties between factors
 // decided by fit_rows_exact); without that it took 80 us when it took 88 with it.
