@@ -19,10 +19,8 @@
 // them, the chain of each token's sums, which the 16 warps per SM do not quite hide.  16 x 32 heads
 // of 128 x 128, 32 tokens: 74 us; 463 us with a launch per token, each reading and writing the
 // state (67 MB).
-// A call of one token is its state's trip through memory: 16 x 32 heads of 128 x 128 16.6 us from
-// HBM (4.0 TB/s; 18.3 us with 8 neighbouring columns per lane, whose accesses took half a sector each)
-// and 14.1 us from L2 (16.8 us), bound by the L1's lookups, as a warp's 16 columns are 64 bytes of a row; a
-// kernel whose warps hold whole rows takes 16.4 and 11.4 us there, and 26.7 us for 4 tokens (19 us here).
+// Calls of one or two tokens, which are little but the state's way through memory, have a kernel of their
+// own (below).
 #include "qs_common.cuh"
 
 namespace qs {
@@ -287,8 +285,141 @@ __global__ void __launch_bounds__(kFpThreads, 4) scan_fp32_kernel(const __grid_c
     }
 }
 
+// ---- a call of few tokens ----------------------------------------------------------------------
+// Such a call is its state's way through memory.  Same CTAs (64 columns of a head, 4 warps), but half a
+// warp holds 256 bytes of a row and a warp's rows lie beside each other, so that a 16-byte access of the warp
+// takes 4 lines of the L1 (16 in the kernel above); the price is an exchange between the warps
+// for each token's sums, three barriers per token.  16 x 32 heads of 128 x 128, one token: 13.6 us from HBM
+// (67 MB, 4.9 TB/s) and 9.0 us from L2; the kernel above 16.6 and 14.1, one CTA of 8 warps to a head 16.4 and 11.4.
+// Two tokens 15.7 and 11.1 (16.9 and 14.7), three 17.2 and 12.9 (17.5 and 15.6), four 19.0 and 14.8 (18.9 and 17.1);
+// 64 x 32 heads, two 53 and 53 (52 and 52), three 58 and 57: hence up to two.  The readouts' error against
+// 64 bits is the kernel above's (8.9e-8 and 8.8e-8 for one token, 9.5e-8 both for two).
+constexpr int kShortTokens = 2;
+
+template <int DK, int ERASE>
+__global__ void __launch_bounds__(kFpThreads, 4) scan_fp32_short_kernel(const __grid_constant__ StepParams p, int dv) {
+    constexpr int RT = DK / 8;   // rows per thread: 8 r + rg
+    __shared__ float4 dakq[DK];  // decay, a (delta rule: k), k, q of the token's rows
+    __shared__ __align__(16) float red[2][4][kCols], us[kCols];
+    __shared__ float wsum[DK / 32];
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, rg = tid >> 4, cl = (tid & 15) * 4;
+    const int parts = dv / kCols;
+    const int bh = blockIdx.x / parts, c0 = (blockIdx.x - bh * parts) * kCols;
+    const int b = bh / p.H, h = bh - b * p.H;
+    const size_t at = (static_cast<size_t>(bh) * DK + rg) * dv + c0 + cl;   // + 8 r dv
+    float2 x[RT][2];
+#pragma unroll
+    for (int r = 0; r < RT; ++r) {
+        const float4 v = *reinterpret_cast<const float4*>(p.dense_in + at + static_cast<size_t>(8 * r) * dv);
+        x[r][0] = make_float2(v.x, v.y);
+        x[r][1] = make_float2(v.z, v.w);
+    }
+#pragma unroll 1
+    for (int t = p.t_begin; t < p.t_end; ++t) {
+        const size_t tok = (static_cast<size_t>(b) * p.T + t) * p.H + h;
+        if (t > p.t_begin) __syncthreads();   // the token before is done with its rows and u
+        float vj = 0.0f, wj = 1.0f;
+        if (tid < kCols) {
+            vj = p.v[tok * dv + c0 + tid];
+            if constexpr (ERASE == kEraseDelta) wj = p.beta[tok];
+            if constexpr (ERASE == kEraseGeneral) wj = p.w_in[tok * dv + c0 + tid];
+        }
+        if (tid < DK) {
+            const float k = p.k[tok * DK + tid], q = p.q[tok * DK + tid];
+            float a = k, rate;
+            if constexpr (ERASE == kEraseGeneral) a = p.a_in[tok * DK + tid];
+            if (p.s_code) {
+                const size_t ch = p.decay_row ? static_cast<size_t>(h) * DK + tid : h;
+                rate = p.s_lut[ch * p.L + min(static_cast<int>(p.s_code[p.decay_row ? tok * DK + tid : tok]), p.L - 1)];
+            } else {
+                rate = p.s[p.decay_row ? tok * DK + tid : tok];
+            }
+            if (!(rate > 0.0f) || !(rate < INFINITY)) raise_status(p.status, QS_DEV_RATE);
+            dakq[tid] = make_float4(expf(-rate), a, k, q);
+            const float kq = warp_sum(k * q);
+            if (lane == 0) wsum[warp] = kq;
+        }
+        __syncthreads();
+        // (four runs of RT / 4 rows summed by halves, so that the sums round no worse than the kernel above's)
+        float2 pp[2], rr[2];
+        auto run = [&](int r0, float2 (&ps)[2], float2 (&rs)[2]) {
+#pragma unroll
+            for (int i = 0; i < RT / 4; ++i) {
+                const int r = r0 + i;
+                const float4 f = dakq[8 * r + rg];
+#pragma unroll
+                for (int c = 0; c < 2; ++c) {
+                    x[r][c] = __fmul2_rn(x[r][c], make_float2(f.x, f.x));
+                    if constexpr (ERASE != kEraseNone)
+                        ps[c] = i == 0 ? __fmul2_rn(x[r][c], make_float2(f.y, f.y)) : __ffma2_rn(x[r][c], make_float2(f.y, f.y), ps[c]);
+                    rs[c] = i == 0 ? __fmul2_rn(x[r][c], make_float2(f.w, f.w)) : __ffma2_rn(x[r][c], make_float2(f.w, f.w), rs[c]);
+                }
+            }
+        };
+#pragma unroll
+        for (int half = 0; half < 2; ++half) {
+            float2 p0[2], r0[2], p1[2], r1[2];
+            run(half * (RT / 2), p0, r0);
+            run(half * (RT / 2) + RT / 4, p1, r1);
+#pragma unroll
+            for (int c = 0; c < 2; ++c) {
+                if constexpr (ERASE != kEraseNone) {
+                    p0[c] = __fadd2_rn(p0[c], p1[c]);
+                    pp[c] = half == 0 ? p0[c] : __fadd2_rn(pp[c], p0[c]);
+                }
+                r0[c] = __fadd2_rn(r0[c], r1[c]);
+                rr[c] = half == 0 ? r0[c] : __fadd2_rn(rr[c], r0[c]);
+            }
+        }
+        // the warp's two halves, then the four warps
+        auto both = [&](float2 v) {
+            return make_float2(v.x + __shfl_xor_sync(kFull, v.x, 16), v.y + __shfl_xor_sync(kFull, v.y, 16));
+        };
+#pragma unroll
+        for (int c = 0; c < 2; ++c) {
+            if constexpr (ERASE != kEraseNone) pp[c] = both(pp[c]);
+            rr[c] = both(rr[c]);
+        }
+        if (lane < 16) {
+            if constexpr (ERASE != kEraseNone)
+                *reinterpret_cast<float4*>(&red[0][warp][cl]) = make_float4(pp[0].x, pp[0].y, pp[1].x, pp[1].y);
+            *reinterpret_cast<float4*>(&red[1][warp][cl]) = make_float4(rr[0].x, rr[0].y, rr[1].x, rr[1].y);
+        }
+        __syncthreads();
+        if (tid < kCols) {
+            float P = 0.0f;
+            if constexpr (ERASE != kEraseNone) P = (red[0][0][tid] + red[0][1][tid]) + (red[0][2][tid] + red[0][3][tid]);
+            const float R = (red[1][0][tid] + red[1][1][tid]) + (red[1][2][tid] + red[1][3][tid]);
+            float kq = wsum[0] + wsum[1];
+            if constexpr (DK == 128) kq += wsum[2] + wsum[3];
+            // as above: u = beta (v - p), w o v - p, or v
+            float u = vj;
+            if constexpr (ERASE == kEraseDelta) u = __fmul_rn(wj, __fsub_rn(vj, P));
+            if constexpr (ERASE == kEraseGeneral) u = __fsub_rn(__fmul_rn(wj, vj), P);
+            us[tid] = u;
+            p.o[tok * dv + c0 + tid] = fmaf(u, kq, R);
+        }
+        __syncthreads();
+        const float4 u = *reinterpret_cast<const float4*>(&us[cl]);
+#pragma unroll
+        for (int r = 0; r < RT; ++r) {
+            const float k = dakq[8 * r + rg].z;
+            x[r][0] = __ffma2_rn(make_float2(k, k), make_float2(u.x, u.y), x[r][0]);
+            x[r][1] = __ffma2_rn(make_float2(k, k), make_float2(u.z, u.w), x[r][1]);
+        }
+    }
+#pragma unroll
+    for (int r = 0; r < RT; ++r)
+        *reinterpret_cast<float4*>(p.dense_out + at + static_cast<size_t>(8 * r) * dv) =
+            make_float4(x[r][0].x, x[r][0].y, x[r][1].x, x[r][1].y);
+}
+
 template <int DK, int ERASE>
 cudaError_t launch_fp32_t(const StepParams& p, int dv, int vec, cudaStream_t stream) {
+    if (p.t_end - p.t_begin <= kShortTokens && (vec & 2)) {
+        scan_fp32_short_kernel<DK, ERASE><<<p.B * p.H * (dv / kCols), kFpThreads, 0, stream>>>(p, dv);
+        return cudaGetLastError();
+    }
     const int smem = static_cast<int>(sizeof(FpSmem<DK, ERASE>));
     cudaError_t e = cudaFuncSetAttribute(scan_fp32_kernel<DK, ERASE>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;

@@ -70,3 +70,12 @@ def test_scan_fp32(qs, dk, dv, erase, rates, t0, t1, pad):
     before = S.clone()
     qs.qstate_scan_fp32(cfg, S, X, t1, t1, o)   # no tokens
     assert torch.equal(S, before)
+
+
+@pytest.mark.parametrize("dk,dv", [(128, 128), (128, 64), (64, 64)])
+@pytest.mark.parametrize("erase", [0, 1, 2])
+@pytest.mark.parametrize("rates", ["row", "head_code"])
+@pytest.mark.parametrize("t0,t1,pad", [(0, 2, 0), (7, 8, 0), (7, 9, 0), (0, 3, 0), (0, 1, 1), (0, 2, 2)])
+def test_few_tokens(qs, dk, dv, erase, rates, t0, t1, pad):
+    """Calls of one or two tokens on an aligned state have a kernel of their own: both sides of that line."""
+    test_scan_fp32(qs, dk, dv, erase, rates, t0, t1, pad)
