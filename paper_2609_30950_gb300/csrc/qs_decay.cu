@@ -51,12 +51,15 @@ constexpr int kMinmaxBlocks = 5;
 constexpr uint32_t kMaxRate = 0x7f7fffffu;   // the largest finite float
 constexpr int codes_blocks(int lm1) { return lm1 <= 3 ? 5 : lm1 <= 7 ? 3 : 2; }
 
-template <int LC, bool ANY>
+// ANYC: with ANY, the most channels (256 or kAnyChannels: the shared extrema are set and read for each);
+// else 0.
+template <int LC, int ANYC>
 __global__ void __launch_bounds__(kDecayThreads, kMinmaxBlocks) decay_minmax_rows_kernel(const float* __restrict__ s, const Walk wk, int L,
                                                                           float* lut, int* status) {
     constexpr int RS = kDecayThreads / LC;
     __shared__ uint4 smn[RS][LC], smx[RS][LC];
-    constexpr int NC = ANY ? kAnyChannels : 4 * LC;
+    constexpr bool ANY = ANYC > 0;
+    constexpr int NC = ANY ? ANYC : 4 * LC;
     __shared__ uint32_t cmn[NC], cmx[NC];
     const int lane = threadIdx.x % LC, sub = threadIdx.x / LC;
     const int chunk = blockIdx.x % wk.chunks;
@@ -118,7 +121,7 @@ __global__ void __launch_bounds__(kDecayThreads, kMinmaxBlocks) decay_minmax_row
     if constexpr (ANY) {
         // the block's values follow one another from a multiple of 1024 on: every nc-th is a channel's
         const long long first = static_cast<long long>(blockIdx.x) * 4 * kDecayThreads;
-        if (nc <= kDecayThreads) {
+        if (ANYC <= kDecayThreads || nc <= kDecayThreads) {
             const int per = kDecayThreads / nc * nc, t = threadIdx.x;
             if (t < per) {
                 uint32_t lo = ~0u, hi = 0u;
@@ -157,7 +160,7 @@ __global__ void __launch_bounds__(kDecayThreads, kMinmaxBlocks) decay_minmax_row
     }
     __syncthreads();
     for (int i = threadIdx.x; i < nc; i += kDecayThreads) {
-        if (cmx[i] == 0u) continue;   // no good rate of this channel here
+        if (ANYC > 256 && cmx[i] == 0u) continue;   // no good rate of this channel here
         float* l = lut + (static_cast<size_t>(chunk) * 4 * LC + i) * L;
         atomicMin(reinterpret_cast<uint32_t*>(l), cmn[i]);
         atomicMax(reinterpret_cast<uint32_t*>(l + L - 1), cmx[i]);
@@ -341,10 +344,11 @@ cudaError_t launch_quant_decay(const float* s, long long count, int nchan, int g
         // of many heads, each block's extrema are as many atomics: 16 samples to a block at least (4096
         // samples of 1000 heads, 4 levels: 30 us without this)
         const long long most = any && nchan > 256 ? std::max(1LL, count / 16) : 1LL << 31;
-#define QS_DM(LC, ANY) decay_minmax_rows_kernel<LC, ANY><<<blocks_of(kMinmaxBlocks, most), kDecayThreads, 0, stream>>>(s, wk, L, lut, status)
-        if (any) QS_DM(32, true);
-        else if (lc == 32) QS_DM(32, false);
-        else QS_DM(16, false);
+#define QS_DM(LC, ANYC) decay_minmax_rows_kernel<LC, ANYC><<<blocks_of(kMinmaxBlocks, most), kDecayThreads, 0, stream>>>(s, wk, L, lut, status)
+        if (any && nchan > 256) QS_DM(32, kAnyChannels);
+        else if (any) QS_DM(32, 256);
+        else if (lc == 32) QS_DM(32, 0);
+        else QS_DM(16, 0);
 #undef QS_DM
     } else {
         // S = a multiple of lcm(nchan, 256) near (SMs x 8) CTAs of 256 threads
