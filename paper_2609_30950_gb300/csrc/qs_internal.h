@@ -93,8 +93,8 @@ struct AllocParams {
     float e1[17];      // 1/k! (FP64 -> FP32) for the expm1 series, k = 1..16
 };
 
-// Launch of a kernel that begins with chain_wait().  early: its CTAs may be placed, and run up to that
-// point, while the launch before it in the stream still runs: the launch's latency and the kernel's
+// Launch of a kernel that begins with chain_wait() or its halves.  early: its CTAs may be placed, and run up
+// to that point, while the launch before it in the stream still runs: the launch's latency and the kernel's
 // start are then behind it (256 write-backs and allocations of one 64 x 64 head: 12.4 -> 9.6 us
 // each; one-prompt prefill 811 -> 730 us).  The chains of a partitioned scan launch without it:
 // CTAs that wait in one chain would hold SMs that another chain's work fills (KDA prefill, 2 chains:
